@@ -132,8 +132,13 @@ typedef struct {
                             0 = none.  Values above 7, and bit 2 without bit 0, are
                             invalid. */
     int32_t s_transform; /* how D_t is applied along s (same result to rounding):
-                            0 auto: for a single curve the form measured fastest on GB300 for its
-                            size: from N_s = 684 on (FFT length >= 4096) a four-step FFT form:
+                            0 auto: from N_s = 64 up to 16384 (FP32 storage) or 8192 (FP64) the
+                            column form, for single curves and batches: one real column per
+                            CTA (FP64 curves of few columns: per cluster of 2 or 4 CTAs), its
+                            sections' differences convolved in registers and shared memory,
+                            fields stored column by column.  Elsewhere, and as the name that
+                            ks_curve_s_form and ks_curve_fft_length give every size, the form
+                            measured fastest among the others: from N_s = 684 on (FFT length >= 4096) a four-step FFT form:
                             in FP32 the clustered one (5) at N_x <= 64 up to N_s = 5462 and at
                             N_x = 128 up to N_s = 2731, else the three-launch one (4); in FP64
                             the clustered one at N_x <= 16 up to N_s = 1366, the one-CTA form
@@ -193,7 +198,7 @@ int32_t ks_version(void);
  * parameters are invalid; ks_last_error() says why).  The workspace holds the
  * spectral state, its s-derivative, the residual, the adjoint, the
  * rational-Chebyshev tables (O(N_s)), the Fourier tables and the FP64
- * reduction buffers: about 6 N_s N storage words in total.  No O(N_s^2)
+ * reduction buffers: about 7 N_s N storage words in total (FP32 storage).  No O(N_s^2)
  * matrix is stored: D_t is generated from an O(N_s) table on the fly. */
 size_t ks_curve_workspace_bytes(const ks_params *p);
 
@@ -202,8 +207,9 @@ size_t ks_curve_workspace_bytes(const ks_params *p);
  * p is invalid (message in ks_last_error). */
 int32_t ks_curve_fft_length(const ks_params *p);
 
-/* The form a single curve with parameters p applies D_t in, as an s_transform
- * code with `auto` resolved: 1 dense, 2 FFT with one CTA per mode, 3 dense on the
+/* The form a size names under the rule above, as an s_transform code with `auto`
+ * resolved among the codes below (where `auto` runs the column form, the code and
+ * ks_curve_fft_length still name the size's other form): 1 dense, 2 FFT with one CTA per mode, 3 dense on the
  * tensor cores, 4 four-step FFT in three launches, 5 four-step FFT in one
  * clustered launch.  -1 when p is invalid (message in ks_last_error). */
 int32_t ks_curve_s_form(const ks_params *p);
@@ -297,7 +303,8 @@ ks_status ks_curve_set_state(ks_curve *c, const void *u_dev, double lambda, doub
  * FFT form) are timed per phase:
  *   phase 0: row phase (f, residual, spatial adjoint, cost reductions)
  *   phase 1: s-phase with the descent update (D_t r, G, u update, |G|^2)
- *   phase 2: s-phase D_t u of the new state;
+ *   phase 2: s-phase D_t u of the new state (none where the update's launch applies it:
+ *            the column form and the clustered four-step form);
  * launches of the persistent step kernel are timed whole (step_*).
  * ks_curve_profile(c, max_steps) starts recording for up to max_steps steps or
  * persistent launches (max_steps = 0 stops and releases the events);
@@ -366,7 +373,9 @@ ks_status ks_batch_get_state(ks_batch *b, int32_t i, void *u_dev);
  *   2. for each transform length F of the four-step curves (the batched FFT form
  *      from F = 1024 on), the split F = F1 F2 of its line transforms: 32 x 32;
  *      64 x 32 or 32 x 64; 64 x 64, 128 x 32 or 32 x 128; 128 x 64 (the kernel
- *      spectrum and twiddles are recomputed for the split);
+ *      spectrum and twiddles are recomputed for the split; none of it applies to curves
+ *      in the column form, for which ks_batch_get_tuning lists the length and the
+ *      default split their sizes name);
  *   3. for dense-form curves with N >= 64, the s-phase tile width: 64 or 32 columns.
  * *chosen (may be NULL) receives the sections per row CTA; ks_batch_get_tuning
  * reports every choice.  Synchronises. */

@@ -18,6 +18,8 @@ namespace {
 
 const int BATCH_GRAPH_STEPS = 16;
 
+constexpr int CM_KEY = 1 << 16;   // row group of column-major curves: N + CM_KEY
+
 struct Group {
     int key;              // N (rows), tile width (dense s-phase) or F (FFT s-phase)
     size_t off;           // offset of the item list in the item area
@@ -40,9 +42,11 @@ struct ks_batch {
     unsigned char *items_dev = nullptr; // item area
     size_t items_cap = 0;
     std::vector<Group> rows, dts;
+    std::vector<Group> ccs;             // (curve, column) items of the column form, one group per length
     std::vector<Group> ffts;            // (curve, mode) items of the FFT-form curves, one group per F
     int impl = 0;                       // full-linear-implicit stepping
     Group imp_prod{}, imp_fin{};        // its items: the two products, the finishing pass
+    std::map<int, int> named;           // column-form curves: the transform length and split their sizes name
     int tile_pref = 0;                  // 0: per-curve default, 32 or 64: forced (autotuner)
     int row_warps = ks::ROWS_WARPS;     // warps per row-phase CTA (two sections each): 4 or 8 (autotuner)
     float tuned_ms = 0.f;               // the autotuner's time of a step with its choice
@@ -61,7 +65,7 @@ void header_sizes(int nb, const ks_params *p, size_t *cv_bytes, size_t *items_by
     for (int i = 0; i < nb; ++i) {
         rows += (p[i].ns + ks::ROWS_PER_CTA - 1) / ks::ROWS_PER_CTA;
         tiles += (size_t)((p[i].ns + ks::DT_BM - 1) / ks::DT_BM) * ((p[i].nx + 31) / 32);
-        modes += p[i].nx / 2;
+        modes += p[i].nx;   // column pairs, or the column form's columns
         if (p[i].scheme == KS_SCHEME_IMPLICIT)   // the increment's products (<= 2 per tile) and finishing pass (<= 8)
             imp += 2 * (size_t)((p[i].nx + 63) / 64) * ((p[i].ns - 1) / 2 / 128 + 1) + 8;
     }
@@ -94,12 +98,18 @@ ks_status build_items(ks_batch *b)
 {
     std::map<int, std::vector<int2>> rows;
     std::map<int, std::vector<int4>> dts;
+    std::map<int, std::vector<int2>> cols;                  // column form: (curve, column) items by length
     std::map<std::pair<int, int>, std::vector<int2>> fft;   // by (F, F1): each group launched with its own shared memory
     for (int i = 0; i < b->nb; ++i) {
         ks::CurveDev &c = b->cv[i];
-        const int rs = 2 * b->row_warps;
+        if (c.cc) c.rsec = ks::cm_sections(c.nx, c.ns, b->prec, 2 * b->row_warps, 0);
+        const int rs = c.cc ? c.rsec : 2 * b->row_warps;
         c.row_blocks = (c.ns + rs - 1) / rs;
-        for (int k = 0; k < c.row_blocks; ++k) rows[c.nx].push_back(make_int2(i, k));
+        for (int k = 0; k < c.row_blocks; ++k) rows[c.nx + (c.cc ? CM_KEY : 0)].push_back(make_int2(i, k));
+        if (c.cc) {
+            for (int col = 0; col < c.W; ++col) cols[c.cc].push_back(make_int2(i, col));
+            continue;
+        }
         if (c.F > 0) {
             for (int jm = 0; jm < c.W / 2; ++jm) fft[std::make_pair(c.F, c.f4b ? c.F1 : 0)].push_back(make_int2(i, jm));
             continue;
@@ -132,6 +142,12 @@ ks_status build_items(ks_batch *b)
     b->ffts.clear();
     for (auto it = fft.rbegin(); it != fft.rend(); ++it) {   // largest F (longest CTAs) first
         b->ffts.push_back({it->first.first, o, (int)it->second.size(), it->first.second});
+        memcpy(host.data() + o, it->second.data(), it->second.size() * sizeof(int2));
+        o += it->second.size() * sizeof(int2);
+    }
+    b->ccs.clear();
+    for (auto it = cols.rbegin(); it != cols.rend(); ++it) {   // longest first
+        b->ccs.push_back({it->first, o, (int)it->second.size()});
         memcpy(host.data() + o, it->second.data(), it->second.size() * sizeof(int2));
         o += it->second.size() * sizeof(int2);
     }
@@ -173,13 +189,28 @@ static cudaError_t launch_fft_group(const ks_batch *b, const Group &g, int mode,
     return ks::launch_sconv_batch(b->prec, g.key, b->cv_dev, items, g.count, mode, discrete, 1, st);
 }
 
+static cudaError_t launch_rows_group(const ks_batch *b, const Group &g, int mode, cudaStream_t st)
+{
+    const int2 *items = (const int2 *)(b->items_dev + g.off);
+    if (g.key >= CM_KEY)
+        return ks::launch_rows_cm_batch(b->prec, g.key - CM_KEY, 2 * b->row_warps, b->cv_dev, items, g.count, mode, st);
+    return ks::launch_rows_batch(b->prec, g.key, b->row_warps, b->cv_dev, items, g.count, mode, st);
+}
+
 ks_status launch_step(ks_batch *b, cudaStream_t st)
 {
     cudaError_t e = cudaSuccess;
     for (const Group &g : b->rows)
-        if (e == cudaSuccess)
-            e = ks::launch_rows_batch(b->prec, g.key, b->row_warps, b->cv_dev, (const int2 *)(b->items_dev + g.off), g.count,
-                                      ks::ROWS_STEP, st);
+        if (e == cudaSuccess) e = launch_rows_group(b, g, ks::ROWS_STEP, st);
+    // the column form: the update and D_t u of the updated state in one launch, unless
+    // the implicit increment comes between them
+    auto cols = [&](int mode, int discrete) {
+        for (const Group &g : b->ccs)
+            if (e == cudaSuccess)
+                e = ks::launch_cc_batch(b->prec, g.key, b->cv_dev, (const int2 *)(b->items_dev + g.off), g.count, mode,
+                                        discrete, 1, st);
+    };
+    cols(b->impl ? ks::GM_GRAD : ks::GM_STEP, b->discrete);
     // the update contraction; for the implicit scheme it writes G, whose increment follows
     const int um = b->impl ? ks::GM_GRAD : ks::GM_UPDATE;
     for (const Group &g : b->dts)
@@ -195,6 +226,7 @@ ks_status launch_step(ks_batch *b, cudaStream_t st)
         e = ks::launch_implicit_batch(b->prec, b->cv_dev, (const int4 *)(b->items_dev + b->imp_prod.off),
                                       b->imp_prod.count, (const int4 *)(b->items_dev + b->imp_fin.off),
                                       b->imp_fin.count, st);
+    if (b->impl) cols(ks::GM_STORE, 0);
     for (const Group &g : b->dts)
         if (e == cudaSuccess)
             e = ks::launch_dt_batch(b->prec, g.key, b->cv_dev, (const int4 *)(b->items_dev + g.off), g.count,
@@ -269,9 +301,7 @@ ks_status eval_all(ks_batch *b)
 {
     cudaError_t e = cudaSuccess;
     for (const Group &g : b->rows)
-        if (e == cudaSuccess)
-            e = ks::launch_rows_batch(b->prec, g.key, b->row_warps, b->cv_dev, (const int2 *)(b->items_dev + g.off), g.count,
-                                      ks::ROWS_EVAL, b->st);
+        if (e == cudaSuccess) e = launch_rows_group(b, g, ks::ROWS_EVAL, b->st);
     if (e != cudaSuccess) return ks::report_error(KS_ECUDA, "batched evaluation: %s", cudaGetErrorString(e));
     return KS_OK;
 }
@@ -366,6 +396,7 @@ ks_status ks_batch_create(int32_t nb, const ks_params *params, const double *u_p
                                              (params[i].symmetry & KS_SYM_SINE) ? 1 : 0);
         b->off.push_back(o);
         b->cv[i] = ks::bind_layout(&params[i], l, base + o);
+        if (l.cc && l.f4b) b->named[l.F] = l.F1;
         o += l.total;
     }
     s = KS_OK;
@@ -574,7 +605,7 @@ ks_status ks_batch_get_tuning(ks_batch *b, ks_batch_tuning *out)
     *out = ks_batch_tuning{};
     out->row_sections = 2 * b->row_warps;
     out->dense_tile = b->tile_pref;
-    std::map<int, int> lens;
+    std::map<int, int> lens = b->named;
     for (int i = 0; i < b->nb; ++i)
         if (b->cv[i].f4b) lens[b->cv[i].F] = b->cv[i].F1;
     for (auto &kv : lens) {

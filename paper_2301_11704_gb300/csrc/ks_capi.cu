@@ -152,10 +152,12 @@ ks_status read_scalars(ks_curve *c, ks::DevScalars *h)
     return KS_OK;
 }
 
-// The clustered four-step form applies the update and D_t u of the updated state
-// in one launch (GM_STEP) at the sizes of f4c_fused; every other form in two.
+// The column form, and the clustered four-step form at the sizes of f4c_fused, apply
+// the update and D_t u of the updated state in one launch (GM_STEP); every other
+// form in two.
 static bool fused_step(const ks_curve *c)
 {
+    if (c->d.cc) return !c->d.impl;
     return c->d.f4c != 0 && !c->d.impl && ks::f4c_fused(c->d.prec, c->d.W, c->d.F);
 }
 
@@ -371,7 +373,7 @@ ks_status ks_curve_create(const ks_params *p, const double *u_plus_host, const d
             r = fail(KS_ENOMEM, "pinned host allocation of the scalars failed");
             break;
         }
-        if (!c->d.xtc && p->ns >= ks::ROWS_TMA_MIN_NS) {
+        if (!c->d.xtc && !c->d.cc && p->ns >= ks::ROWS_TMA_MIN_NS) {
             const cudaError_t e = ks::make_row_maps(c->d, &c->rmaps);
             if (e != cudaSuccess) {
                 r = fail(KS_ECUDA, "encoding the row phase's tensor maps failed: %s", cudaGetErrorString(e));
@@ -515,7 +517,9 @@ ks_status ks_curve_descend_async(ks_curve *c, int64_t nsteps, double tol)
     if (!std::isfinite(tol)) return fail(KS_EINVAL, "tol must be finite");
     DeviceGuard g(c->device);
     if (!g.ok) return fail(KS_ECUDA, "cannot select the curve's device");
-    return enqueue_steps(c, nsteps, tol);
+    s = enqueue_steps(c, nsteps, tol);
+    if (s == KS_OK && c->d.defer && nsteps > 0) KS_CUDA(ks::launch_cc_finish(c->d, c->st));
+    return s;
 }
 
 ks_status ks_curve_descend(ks_curve *c, int64_t nsteps, double tol, int64_t *steps_done, double *J, double *J_arc)

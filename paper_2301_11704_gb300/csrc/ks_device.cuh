@@ -13,8 +13,9 @@
 
 namespace ks {
 
+// aligned to its size: one 8- or 16-byte access per value
 template <typename T>
-struct cpx {
+struct alignas(2 * sizeof(T)) cpx {
     T x, y;
 };
 
@@ -33,6 +34,7 @@ __device__ __forceinline__ cpx<T> cmul(cpx<T> a, cpx<T> b)
 // no CTA leaves before it.  No kernel triggers its successor early: successor
 // CTAs parked on the SMs during a whole kernel slowed graph replay (measured).
 // A no-op for a kernel launched without the attribute.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Arrival of a CTA at a grid-wide last-CTA reduction, after the CTA has written
@@ -388,6 +390,31 @@ __device__ __forceinline__ int rows_finish(const CurveDev &c, int mode, int nblk
     }
     __syncthreads();
     return go;
+}
+
+// Deferred form (CurveDev::defer): the sum of the last update's |G|^2 partials (one per
+// warp of each column, c.g2_parts) in a fixed order, in a CTA of its own (nt threads, at
+// most 256) beside the next row phase.
+__device__ __forceinline__ void finish_g2(const CurveDev &c, int nt)
+{
+    __shared__ double part[8];
+    DevScalars *sc = c.sc;
+    if (!sc->g2_pending) return;
+    const int tid = threadIdx.x;
+    if (nt > 256) nt = 256;
+    double t = 0.0;
+    if (tid < nt) {
+        for (int b = tid; b < c.g2_parts; b += nt) t += __ldcg(c.tile + b);
+        t = warp_sum(t);
+        if ((tid & 31) == 0) part[tid >> 5] = t;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        t = 0.0;
+        for (int w = 0; w < nt / 32; ++w) t += part[w];
+        sc->G2 = c.L * t;
+        sc->g2_pending = 0;
+    }
 }
 
 // Shared-memory tiles of the row phase's TMA loads: U and D_t U rows of the CTA,

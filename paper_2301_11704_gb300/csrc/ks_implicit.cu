@@ -345,19 +345,22 @@ constexpr int IM_BM = 128, IM_BN = 64, IM_BK = 16, IM_THREADS = 256, IM_TM = 8, 
 template <typename T>
 struct ImSmem {
     __align__(16) T As[IM_BK][IM_BM];
-    __align__(16) T Bs[IM_BK][IM_BN];
+    __align__(16) T Bs[IM_BK][IM_BN + 4];   // (B tiles of column-major operands are written k-fastest)
 };
 
 // acc[i][l] += sum_{k in [kb, ke)} A[r0 + 8 ty + i][k] B(k, c0 + 4 tx + l);
-// A row-major (nrows x lda), B(k, col) from `loadb` (called for k < ke, col < ncols).
+// A row-major (nrows x lda), B(k, col) from `loadb` (called for k < ke, col < ncols),
+// contiguous in k (kfast) or in col.
 template <typename T, typename LoadB>
 __device__ __forceinline__ void im_tile(ImSmem<T> &sm, const T *A, int nrows, int lda, int r0, int kb, int ke, int c0,
-                                        int ncols, LoadB loadb, T (&acc)[IM_TM][IM_TN])
+                                        int ncols, bool kfast, LoadB loadb, T (&acc)[IM_TM][IM_TN])
 {
     constexpr int AL = IM_BM * IM_BK / IM_THREADS, BL = IM_BK * IM_BN / IM_THREADS;
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int ar = tid >> 1, ak = (tid & 1) * AL;   // A: a row and 8 consecutive k per thread
     T ra[AL], rb[BL];
+    auto bk = [&](int q) { const int e = tid + q * IM_THREADS; return kfast ? e % IM_BK : e / IM_BN; };
+    auto bc = [&](int q) { const int e = tid + q * IM_THREADS; return kfast ? e / IM_BK : e % IM_BN; };
     auto fetch = [&](int k0) {
         const bool rok = r0 + ar < nrows;
         const T *arow = A + (size_t)(r0 + ar) * lda;
@@ -368,7 +371,7 @@ __device__ __forceinline__ void im_tile(ImSmem<T> &sm, const T *A, int nrows, in
         }
 #pragma unroll
         for (int q = 0; q < BL; ++q) {
-            const int e = tid + q * IM_THREADS, k = k0 + e / IM_BN, col = c0 + e % IM_BN;
+            const int k = k0 + bk(q), col = c0 + bc(q);
             rb[q] = (k < ke && col < ncols) ? loadb(k, col) : T(0);
         }
     };
@@ -379,10 +382,7 @@ __device__ __forceinline__ void im_tile(ImSmem<T> &sm, const T *A, int nrows, in
 #pragma unroll
         for (int q = 0; q < AL; ++q) sm.As[ak + q][ar] = ra[q];
 #pragma unroll
-        for (int q = 0; q < BL; ++q) {
-            const int e = tid + q * IM_THREADS;
-            sm.Bs[e / IM_BN][e % IM_BN] = rb[q];
-        }
+        for (int q = 0; q < BL; ++q) sm.Bs[bk(q)][bc(q)] = rb[q];
         __syncthreads();
         if (k0 + IM_BK < ke) fetch(k0 + IM_BK);
 #pragma unroll
@@ -429,17 +429,20 @@ __device__ __forceinline__ void imp_fwd_body(ImSmem<T> &sm, const CurveDev &c, i
     for (int i = 0; i < IM_TM; ++i)
 #pragma unroll
         for (int l = 0; l < IM_TN; ++l) acc[i][l] = T(0);
+    const size_t ms = c.ms, cs = c.cs;
     if (p == 0)
-        im_tile<T>(sm, A, np, np, r0, kb, ke, c0, N, [&](int k, int col) -> T {
-            return k < h ? r2 * (G[(size_t)(1 + k) * N + col] + G[(size_t)(M - k) * N + col]) : G[(size_t)(1 + h) * N + col];
+        im_tile<T>(sm, A, np, np, r0, kb, ke, c0, N, ms == 1, [&](int k, int col) -> T {
+            const T *g = G + col * cs;
+            return k < h ? r2 * (g[(1 + k) * ms] + g[(M - k) * ms]) : g[(1 + h) * ms];
         }, acc);
     else
-        im_tile<T>(sm, A, np, np, r0, kb, ke, c0, N, [&](int k, int col) -> T {
-            return r2 * (G[(size_t)(1 + k) * N + col] - G[(size_t)(M - k) * N + col]);
+        im_tile<T>(sm, A, np, np, r0, kb, ke, c0, N, ms == 1, [&](int k, int col) -> T {
+            const T *g = G + col * cs;
+            return r2 * (g[(1 + k) * ms] - g[(M - k) * ms]);
         }, acc);
     const T lam = (T)sc->lambda, dtau = (T)sc->dtau, tl = T(2.0 * M_PI / c.L);
     const double *mu = c.imu + (p ? ne : 0);
-    T *out = (T *)c.isc + (size_t)sp * M * N + (p ? (size_t)ne * N : 0);
+    T *out = (T *)c.isc + (size_t)sp * M * N + (p ? (size_t)ne * c.ims : 0);
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
 #pragma unroll
     for (int i = 0; i < IM_TM; ++i) {
@@ -451,7 +454,7 @@ __device__ __forceinline__ void imp_fwd_body(ImSmem<T> &sm, const CurveDev &c, i
             const int col = c0 + IM_TN * tx + l;
             if (col >= N) continue;
             const T kw = tl * (T)(col >> 1), a = kw * kw * kw * kw - kw * kw;
-            out[(size_t)r * N + col] = dtau / (T(1) + dtau * (a * a - lm)) * acc[i][l];
+            out[(size_t)r * c.ims + (size_t)col * c.ics] = dtau / (T(1) + dtau * (a * a - lm)) * acc[i][l];
         }
     }
 }
@@ -468,7 +471,7 @@ __device__ __forceinline__ void imp_back_body(ImSmem<T> &sm, const CurveDev &c, 
     if (r0 >= np) return;
     int kb, ke;
     im_chunk(np, splits, sp, kb, ke);
-    const size_t off = p ? (size_t)ne * N : 0, stride = (size_t)M * N;
+    const size_t off = p ? (size_t)ne * c.ims : 0, stride = (size_t)M * N;
     const T *Pf = (const T *)c.isc;
     const T *A = (const T *)c.iv + (p ? (size_t)ne * ne : 0);
     T acc[IM_TM][IM_TN];
@@ -476,8 +479,8 @@ __device__ __forceinline__ void imp_back_body(ImSmem<T> &sm, const CurveDev &c, 
     for (int i = 0; i < IM_TM; ++i)
 #pragma unroll
         for (int l = 0; l < IM_TN; ++l) acc[i][l] = T(0);
-    im_tile<T>(sm, A, np, np, r0, kb, ke, c0, N, [&](int k, int col) -> T {
-        const T *y = Pf + off + (size_t)k * N + col;
+    im_tile<T>(sm, A, np, np, r0, kb, ke, c0, N, c.ims == 1, [&](int k, int col) -> T {
+        const T *y = Pf + off + (size_t)k * c.ims + (size_t)col * c.ics;
         T t = y[0];
         for (int q = 1; q < splits_f; ++q) t += y[q * stride];
         return t;
@@ -491,7 +494,7 @@ __device__ __forceinline__ void imp_back_body(ImSmem<T> &sm, const CurveDev &c, 
 #pragma unroll
         for (int l = 0; l < IM_TN; ++l) {
             const int col = c0 + IM_TN * tx + l;
-            if (col < N) out[(size_t)r * N + col] = acc[i][l];
+            if (col < N) out[(size_t)r * c.ims + (size_t)col * c.ics] = acc[i][l];
         }
     }
 }
@@ -509,18 +512,21 @@ __device__ __forceinline__ void imp_finish_body(const CurveDev &c, int bx, int n
     const T r2 = T(0.70710678118654752440);
     const long total = (long)ne * N;
     for (long e = bx * (long)IM_THREADS + threadIdx.x; e < total; e += (long)nbx * IM_THREADS) {
-        const int a = (int)(e / N), col = (int)(e % N);
+        // along the fields' contiguous direction
+        const int a = c.ms == 1 ? (int)(e % ne) : (int)(e / N), col = c.ms == 1 ? (int)(e / ne) : (int)(e % N);
         if (!col_allowed(col, c.sym)) continue;
         T de = T(0), dd = T(0);
+        const T *pb = Pb + (size_t)a * c.ims + (size_t)col * c.ics;
         for (int q = 0; q < splits; ++q) {
-            de += Pb[q * stride + (size_t)a * N + col];
-            if (a < h) dd += Pb[q * stride + (size_t)(ne + a) * N + col];
+            de += pb[q * stride];
+            if (a < h) dd += pb[q * stride + (size_t)ne * c.ims];
         }
+        T *u = U + (size_t)col * c.cs;
         if (a < h) {
-            U[(size_t)(1 + a) * N + col] += r2 * (de + dd);
-            U[(size_t)(M - a) * N + col] += r2 * (de - dd);
+            u[(size_t)(1 + a) * c.ms] += r2 * (de + dd);
+            u[(size_t)(M - a) * c.ms] += r2 * (de - dd);
         } else {
-            U[(size_t)(1 + h) * N + col] += de;
+            u[(size_t)(1 + h) * c.ms] += de;
         }
     }
     if (!last_cta_arrive(&sc->cnt_gemm, (unsigned)nbx, am_last)) return;

@@ -168,7 +168,9 @@ __global__ void __launch_bounds__(IT_THREADS, 1) k_imp_tc(CurveDev c, int splits
 
     const int Nn = c.nx;
     const float *G = (const float *)c.G;
-    const float *Y = (const float *)c.isc + (p ? (size_t)ne * Nn : 0);
+    const float *Y = (const float *)c.isc + (p ? (size_t)ne * c.ims : 0);
+    // strides of the B source: G's fields, or the forward partials
+    const size_t rs = FWD ? c.ms : c.ims, cs = FWD ? c.cs : c.ics;
     const float r2 = 0.70710678118654752440f;
     // B chunk q: units (col, k-block of 8) of 8 values, UPT per thread.  `fetch`
     // issues every load of a chunk at once (rows and predicates computed first,
@@ -186,8 +188,8 @@ __global__ void __launch_bounds__(IT_THREADS, 1) k_imp_tc(CurveDev c, int splits
                 const bool v = u < UNITS && k < np;
                 const int ra = FWD ? 1 + k : k;
                 const int rb = (p == 0 && k >= h) ? ra : M - k;   // the mirror row (odd M: the middle alone)
-                xa[j][e] = v ? Bsrc[(size_t)ra * Nn + col] : 0.f;
-                xb[j][e] = (FWD && v) ? G[(size_t)rb * Nn + col] : 0.f;
+                xa[j][e] = v ? Bsrc[ra * rs + col * cs] : 0.f;
+                xb[j][e] = (FWD && v) ? G[rb * rs + col * cs] : 0.f;
             }
         }
     };
@@ -286,8 +288,8 @@ __global__ void __launch_bounds__(IT_THREADS, 1) k_imp_tc(CurveDev c, int splits
     const int r = rt * IT_M + lrow;
     const bool ok = !*vbad && r < np;   // an empty K range (nq = 0) writes zeros
     const size_t stride = (size_t)M * Nn;
-    float *out = (float *)c.isc + (size_t)(FWD ? sp : c.isplits + sp) * stride + (p ? (size_t)ne * Nn : 0) +
-                 (size_t)r * Nn;
+    float *out = (float *)c.isc + (size_t)(FWD ? sp : c.isplits + sp) * stride + (p ? (size_t)ne * c.ims : 0) +
+                 (size_t)r * c.ims;
     const float lam = (float)sc->lambda, dtau = (float)sc->dtau, tl = (float)(2.0 * M_PI / c.L);
     const float lm = FWD && ok ? lam * lam * (float)c.imu[(p ? ne : 0) + r] : 0.f;
 #pragma unroll 1
@@ -304,6 +306,11 @@ __global__ void __launch_bounds__(IT_THREADS, 1) k_imp_tc(CurveDev c, int splits
                 const float kw = tl * (float)(col >> 1), a = kw * kw * kw * kw - kw * kw;
                 y[e] *= dtau / (1.f + dtau * (a * a - lm));
             }
+        }
+        if (c.ics != 1) {   // column-major partials: coalesced over the lanes' rows
+#pragma unroll
+            for (int e = 0; e < 16; ++e) out[(size_t)(c0 + e) * c.ics] = y[e];
+            continue;
         }
 #pragma unroll
         for (int e = 0; e < 16; e += 4)

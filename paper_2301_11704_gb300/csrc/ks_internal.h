@@ -109,6 +109,29 @@ inline int fft4h_size(int ns, int fmin = F4_FMIN)
     return F <= F4_FMAX ? F : 0;
 }
 
+// Length of the column form (ks_colconv.cu: one real column per CTA, right-angle
+// convolution modulo x^L = i, column-major fields): the smallest power of two
+// >= max(N_s, 128), up to what one CTA's shared memory holds; 0 above, and below
+// CC_MIN_NS sections (the other forms' sums are as short as its transform there).
+constexpr int CC_LMAX_F32 = 16384, CC_LMAX_F64 = 8192, CC_MIN_NS = 64;
+inline int cc_size(int ns, int prec)
+{
+    if (ns < CC_MIN_NS) return 0;
+    int L = 128;
+    while (L < ns) L <<= 1;
+    return L <= (prec ? CC_LMAX_F32 : CC_LMAX_F64) ? L : 0;
+}
+// CTAs per column of a single curve: the split form in FP64 where a CTA per column
+// leaves SMs idle (each column is bound by the FP64 pipes of its SM), with classes of
+// 256 to 4096 frequencies.
+inline int cc_cluster(int L, int w, int prec)
+{
+    if (prec) return 1;
+    if (w <= 38 && L >= 1024) return 4;
+    return w <= 76 && L >= 512 ? 2 : 1;
+}
+// words between two columns of a column-major field: whole 128-byte lines
+inline int cc_pitch(int ns) { return (ns + 31) & ~31; }
 // Form of the s-contraction: dense, FFT with one CTA per mode, four-step FFT in
 // three launches, four-step FFT in one clustered launch.
 enum SForm { SF_DENSE = 0, SF_FFT1 = 1, SF_FFT4 = 2, SF_FFT4C = 3 };
@@ -185,6 +208,8 @@ struct DevScalars {
                                         // cycles; < 0: give up at once, a test of the error path)
     unsigned int cnt_rows, cnt_gemm;    // arrival counters of the last-CTA reductions
     unsigned long long bar;             // arrivals at the persistent step's grid barriers
+    int decided;                        // deferred form: 0 undecided, 1 the step is applied, 2 it is not
+    int g2_pending;                     // deferred form: the last update's |G|^2 partials are not summed yet
 };
 
 // Cycles a kernel's first bounded wait may spin for this curve (the waits that
@@ -228,6 +253,11 @@ struct Layout {
     size_t off_ivtc;                   // V^-1 and V as tensor-core operands
     int ivtc;                          // 1: that region exists (single curves, FP32 storage, N >= 32)
     int isplits;                       // K chunks they hold
+    int single;                        // a single curve's layout (0: batched)
+    int ccl;
+    int cc, pitch, rsec;               // column form (cc: its length L, 0: none): column pitch in words,
+                                       // sections per row-phase CTA
+    size_t off_cctw, off_ccs, off_ccr, off_ccx, off_wt, off_twdf;   // its tables; set-up scratch
     int hs;                            // sine storage (odd sections): rows of N/2 words, Im u^_j at j
     int w;                             // stored words per section: N, or N/2 with sine storage
 };
@@ -278,6 +308,23 @@ struct CurveDev {
     double *w;
     void *twid, *twid64, *kj, *aj, *prec_imex;
     double *ends, *pert;
+    // column form (ks_colconv.cu, ks_rows_cm.cu): its length L (0: another form, row-major
+    // fields).  Fields are [W][pitch] words: section m of column col at col * pitch + m.
+    int cc, pitch, rsec;
+    int ccl;                  // CTAs per column: 1, or the cluster of the split form
+    int ms, cs;               // words between two sections and between two columns of a field, in either layout
+    // Deferred reductions (single column-form curves, IMEX): a step's row phase leaves its
+    // row_parts FP64 partials to the contraction, where one CTA sums them and takes the
+    // convergence decision beside the others' first transform; the |G|^2 partials are
+    // summed beside the next row phase (or by launch_cc_finish); lambda_next is the
+    // current lambda from the contraction on.
+    int defer, row_parts, g2_parts;
+    int ims, ics;             // the same of the implicit step's partials (rows of M, columns of N)
+    void *cctw, *ccs;         // twiddles; spectra (T_k, H_k) / L, L pairs of complex values
+    void *ccr;                // row scales -sin^2(theta_j) / S
+    void *ccx;                // set-up scratch: 2 L FP64 complex values
+    void *wt;                 // quadrature weights in the storage type (FP64: w itself)
+    void *twdf;               // FP32 storage: e^(-2 pi i k / N), k < N / 2, as double-float pairs
     DevScalars *sc;
     const RowMaps *rowmaps;   // host pointer: U and D tile maps of a single curve's row phase (else null)
 };
@@ -380,6 +427,27 @@ inline int f4b_splits(int F, int prec, int (&F1s)[3])
     }
     return n;
 }
+
+// Column form (ks_colconv.cu; c.cc set): twiddle entries of a length, set-up of its
+// tables, the s-contraction in the modes of launch_dt (GM_STEP: the update and
+// D_t u of the updated state), and over the (curve, column) items of a batch.
+size_t cc_twiddles(int L, int prec, int cs);
+int cc_warps(int L, int prec, int cs);   // of a column's CTAs
+cudaError_t launch_setup_cc(const CurveDev &c, cudaStream_t st);
+cudaError_t launch_cc(const CurveDev &c, int mode, int discrete, int gate, cudaStream_t st);
+// Deferred form: the |G|^2 of the last update and its lambda, for calls that end with an update.
+cudaError_t launch_cc_finish(const CurveDev &c, cudaStream_t st);
+cudaError_t launch_cc_batch(int prec, int L, const CurveDev *cv, const int2 *items, int nitems, int mode, int discrete,
+                            int gate, cudaStream_t st);
+// Its x-direction kernels on column-major fields (ks_rows_cm.cu).
+// sections per CTA that the row phase is built for: `want` or the next larger
+int cm_sections(int nx, int ns, int prec, int want, int single);
+cudaError_t launch_rows_cm(const CurveDev &c, int mode, cudaStream_t st, StepArm arm);
+cudaError_t launch_rows_cm_batch(int prec, int N, int sec, const CurveDev *cv, const int2 *items, int nitems, int mode,
+                                 cudaStream_t st);
+cudaError_t launch_row_fwd_x_cm(const CurveDev &c, void *spec, cudaStream_t st);
+cudaError_t launch_row_fwd_cm(const CurveDev &c, const void *phys, void *spec, cudaStream_t st);
+cudaError_t launch_row_inv_cm(const CurveDev &c, const void *spec, void *phys, int scale_mode, cudaStream_t st);
 
 // Split-BF16 tensor-core row phase (ks_rows_tc.cu; c.xtc set): bytes of its DFT
 // matrices, their set-up, and the row phase with the modes of launch_rows.

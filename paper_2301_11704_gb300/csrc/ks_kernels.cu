@@ -80,7 +80,17 @@ Layout make_layout(int ns, int nx, int prec, int allow_split, int bn, int s_tran
         l.f4c = (form == SF_FFT4C && f4c_fits(prec, l.F1, l.F2)) ? F4C_CS : 0;
         l.f4b = batched_f4 ? 1 : 0;
     }
-    size_t field = al256((size_t)ns * w * b);
+    // under `auto` the column form runs in place of whatever form the size resolves to
+    // above; that form and its length keep naming the size in ks_curve_s_form and
+    // ks_curve_fft_length
+    l.cc = (s_transform == 0 && !persistent) ? cc_size(ns, prec) : 0;
+    l.pitch = cc_pitch(ns);
+    l.single = allow_split;
+    l.ccl = l.cc && allow_split ? cc_cluster(l.cc, w, prec) : 1;
+    // sections per row-phase CTA: fewer where the curve has few sections (the FP64 work,
+    // and latency, want every SM), 64-byte runs of a column where it has many
+    l.rsec = l.cc ? cm_sections(nx, ns, prec, prec ? (ns >= 2048 ? 16 : 8) : (ns >= 2048 ? 8 : 4), allow_split) : 0;
+    size_t field = l.cc ? al256((size_t)w * l.pitch * b) : al256((size_t)ns * w * b);
     // tiling and split of the s-contraction (over the w stored columns)
     l.bn = bn ? bn : (w >= 64 ? 64 : 32);
     l.tiles_r = (ns + DT_BM - 1) / DT_BM;
@@ -98,6 +108,7 @@ Layout make_layout(int ns, int nx, int prec, int allow_split, int bn, int s_tran
     l.kchunk = kc;
     l.ksplit = (ns + kc - 1) / kc;
     l.row_blocks = (ns + ROWS_PER_CTA - 1) / ROWS_PER_CTA;
+    if (l.cc) l.row_blocks = (ns + l.rsec - 1) / l.rsec;
     // tensor-core form of the dense contraction: FP32 storage, single curves,
     // asked for (s_transform 3) or picked by the measured rule (auto)
     if (prec && allow_split && !hs && l.F == 0 && (s_transform == 3 || (s_transform == 0 && tc_preferred(ns, nx)))) {
@@ -123,9 +134,10 @@ Layout make_layout(int ns, int nx, int prec, int allow_split, int bn, int s_tran
     l.off_G = off; off += field;
     l.off_X = off; off += al256((size_t)ns * nx * 8);   // physical scratch, always FP64
     l.off_rowsc = off; off += al256((size_t)ns * 4 * 8);
-    l.off_bpart = off; off += al256((size_t)l.row_blocks * 5 * 8);
+    l.off_bpart = off; off += al256((size_t)((ns + 3) / 4) * 5 * 8);
     size_t ntile = (size_t)tiles_max * DT_MAX_SPLIT;                   // either contraction form
     if (l.f4 && ntile < (size_t)(l.F2 / 8) * (w / 2)) ntile = (size_t)(l.F2 / 8) * (w / 2);   // four-step CTAs
+    if (l.cc && ntile < (size_t)w * cc_warps(l.cc, prec, l.ccl)) ntile = (size_t)w * cc_warps(l.cc, prec, l.ccl);
     l.off_tile = off; off += al256(ntile * 8);
     l.off_tcnt = off; off += al256((size_t)tiles_max * 4);
     // the persistent step's split partials and per-CTA |G|^2 partials (single
@@ -148,11 +160,18 @@ Layout make_layout(int ns, int nx, int prec, int allow_split, int bn, int s_tran
     l.off_ends = off; off += al256((size_t)2 * nx * 8);
     l.off_pert = off; off += al256((size_t)(nx + MAX_PERT + MAX_PERT * nx) * 8);
     l.off_sc = off; off += al256(sizeof(DevScalars));
-    l.off_chat = off; off += l.F ? al256((size_t)l.F * 2 * b * (l.f4h ? 2 : 1)) : 0;
-    l.off_ftw = off; off += l.F ? al256((size_t)l.F * (l.f4 ? 3 : 1) * 2 * b) : 0;   // four-step: + step twiddles
+    l.off_cctw = off; off += l.cc ? al256(cc_twiddles(l.cc, prec, l.ccl) * 2 * b) : 0;
+    l.off_ccs = off; off += l.cc ? al256((size_t)l.cc * 4 * b) : 0;
+    l.off_ccr = off; off += l.cc ? al256((size_t)ns * b) : 0;
+    l.off_ccx = off; off += l.cc ? al256((size_t)l.cc * 2 * 16) : 0;
+    l.off_wt = off; off += (l.cc && prec) ? al256((size_t)ns * b) : 0;
+    l.off_twdf = off; off += (l.cc && prec) ? al256((size_t)(nx / 2) * 16) : 0;
+    const bool ff = l.F && !l.cc;
+    l.off_chat = off; off += ff ? al256((size_t)l.F * 2 * b * (l.f4h ? 2 : 1)) : 0;
+    l.off_ftw = off; off += ff ? al256((size_t)l.F * (l.f4 ? 3 : 1) * 2 * b) : 0;   // four-step: + step twiddles
     // the three-launch form's scratch (also the FP64 set-up scratch, 32 F bytes);
     // the one-CTA-per-mode variant needs the set-up's only
-    l.off_f4s = off; off += l.f4 ? al256(l.f4b ? (size_t)32 * l.F : (size_t)(w / 2) * l.F * 2 * b) : 0;
+    l.off_f4s = off; off += (l.f4 && !l.cc) ? al256(l.f4b ? (size_t)32 * l.F : (size_t)(w / 2) * l.F * 2 * b) : 0;
     // the split-BF16 row phase's DFT matrices
     l.xtc = xtc;
     l.off_xdft = off; off += xtc ? al256(xdft_bytes(nx)) : 0;
@@ -202,22 +221,40 @@ CurveDev bind_layout(const ks_params *p, const Layout &l, void *base)
     d.ksplit = l.ksplit;
     d.kchunk = l.kchunk;
     d.row_blocks = l.row_blocks;
-    d.F = l.F;
+    d.cc = l.cc;
+    d.pitch = l.pitch;
+    d.rsec = l.rsec;
+    d.defer = l.cc && !l.impl && l.single;
+    d.g2_parts = l.cc ? l.w * cc_warps(l.cc, d.prec, l.ccl) : 0;
+    d.ccl = l.ccl;
+    d.row_parts = l.xtc ? (p->ns + 127) / 128 : l.row_blocks;
+    d.ms = l.cc ? 1 : l.w;
+    d.cs = l.cc ? l.pitch : 1;
+    d.ims = l.cc ? 1 : p->nx;
+    d.ics = l.cc ? p->ns - 2 : 1;
+    d.cctw = b + l.off_cctw;
+    d.ccs = b + l.off_ccs;
+    d.ccr = b + l.off_ccr;
+    d.ccx = b + l.off_ccx;
+    d.wt = d.prec ? (void *)(b + l.off_wt) : (void *)(b + l.off_w);
+    d.twdf = b + l.off_twdf;
+    const bool ff = l.F && !l.cc, f4 = l.f4 && !l.cc;   // a form of its own, not the column form
+    d.F = ff ? l.F : 0;
     d.tc = l.tc;
     d.tc_bn = l.tc_bn;
     d.tc_tiles_r = l.tc_tiles_r;
     d.tc_tiles_c = l.tc_tiles_c;
     d.tc_ksplit = l.tc_ksplit;
     d.tc_kchunk = l.tc_kchunk;
-    d.chat = l.F ? (void *)(b + l.off_chat) : nullptr;
-    d.ftw = l.F ? (void *)(b + l.off_ftw) : nullptr;
-    d.f4s = l.f4 ? (void *)(b + l.off_f4s) : nullptr;
-    d.f4 = l.f4;
+    d.chat = ff ? (void *)(b + l.off_chat) : nullptr;
+    d.ftw = ff ? (void *)(b + l.off_ftw) : nullptr;
+    d.f4s = f4 ? (void *)(b + l.off_f4s) : nullptr;
+    d.f4 = f4 ? 1 : 0;
     d.F1 = l.F1;
     d.F2 = l.F2;
-    d.f4c = l.f4c;
-    d.f4b = l.f4b;
-    d.f4h = l.f4h;
+    d.f4c = f4 ? l.f4c : 0;
+    d.f4b = f4 ? l.f4b : 0;
+    d.f4h = f4 ? l.f4h : 0;
     d.xtc = l.xtc;
     d.xdft = l.xtc ? (void *)(b + l.off_xdft) : nullptr;
     d.impl = l.impl;
@@ -286,6 +323,9 @@ __global__ void k_setup(CurveDev c, double dtau)
             sincospi(2.0 * (double)i / (double)c.nx, &s, &co);
             twid[i] = {(T)co, (T)(-s)};
             ((cpx<double> *)c.twid64)[i] = {co, -s};
+            if (c.cc && c.prec)
+                ((float4 *)c.twdf)[i] = make_float4((float)co, (float)(co - (double)(float)co), (float)(-s),
+                                                    (float)(-s - (double)(float)(-s)));
             double k = 2.0 * M_PI * (double)i / c.L;
             double a = k * k * k * k - k * k;
             kj[i] = (T)k;
@@ -1154,6 +1194,7 @@ cudaError_t launch_setup(const CurveDev &c, double dtau, cudaStream_t st)
     else k_setup<double><<<grid, 256, 0, st>>>(c, dtau);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && c.xtc) e = launch_setup_xdft(c, st);
+    if (e == cudaSuccess && c.cc) return launch_setup_cc(c, st);
     if (e != cudaSuccess || c.F == 0) return e;
     if (c.f4) return launch_setup_f4(c, st);
     const int g2 = (c.F + 255) / 256;
@@ -1223,24 +1264,28 @@ cudaError_t launch_widen(const CurveDev &c, const void *in, cudaStream_t st)
 
 cudaError_t launch_row_fwd_x(const CurveDev &c, void *spec, int keep_ends, cudaStream_t st)
 {
+    if (c.cc) return launch_row_fwd_x_cm(c, spec, st);   // (both callers of the column form transform every row)
     return c.prec ? row_fwd_t<double, double, float>(c, c.X, spec, keep_ends, st)
                   : row_fwd_t<double, double, double>(c, c.X, spec, keep_ends, st);
 }
 
 cudaError_t launch_row_fwd(const CurveDev &c, const void *phys, void *spec, cudaStream_t st)
 {
+    if (c.cc) return launch_row_fwd_cm(c, phys, spec, st);
     return c.prec ? row_fwd_t<float, dfloat, float>(c, phys, spec, 0, st)
                   : row_fwd_t<double, double, double>(c, phys, spec, 0, st);
 }
 
 cudaError_t launch_row_inv(const CurveDev &c, const void *spec, void *phys, int scale_mode, cudaStream_t st)
 {
+    if (c.cc) return launch_row_inv_cm(c, spec, phys, scale_mode, st);
     return c.prec ? row_inv_t<float>(c, spec, phys, scale_mode, st) : row_inv_t<double>(c, spec, phys, scale_mode, st);
 }
 
 cudaError_t launch_rows(const CurveDev &c, int mode, cudaStream_t st, StepArm arm)
 {
     if (c.xtc) return launch_rows_tc(c, mode, st, arm);
+    if (c.cc) return launch_rows_cm(c, mode, st, arm);
     return c.prec ? rows_t<float>(c, mode, st, arm) : rows_t<double>(c, mode, st, arm);
 }
 
@@ -1280,6 +1325,7 @@ cudaError_t launch_sconv_batch(int prec, int F_max, const CurveDev *cv, const in
 
 cudaError_t launch_dt(const CurveDev &c, int mode, int discrete, int gate, cudaStream_t st, cudaEvent_t *pass_ev)
 {
+    if (c.cc) return launch_cc(c, mode, discrete, gate, st);
     if (c.f4b) return launch_f4b(c, mode, discrete, gate, st);
     if (c.f4) return launch_f4(c, mode, discrete, gate, st, pass_ev);
     if (c.F > 0) return c.prec ? launch_sconv_t<float>(c, mode, discrete, gate, st)

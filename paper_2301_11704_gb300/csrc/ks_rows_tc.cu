@@ -107,23 +107,38 @@ __device__ __forceinline__ void put_split(unsigned char *stage, int A_PART, int 
     }
 }
 
-__device__ __forceinline__ void ld_half(const float *p, float (&v)[XT_HV])
+// XT_HV consecutive words of a section: in row-major fields four 16-byte loads, in
+// column-major ones (CM; cs: the column pitch) a word per column, coalesced over
+// the warp's 32 sections.
+template <bool CM>
+__device__ __forceinline__ void ld_half(const float *p, size_t cs, float (&v)[XT_HV])
 {
+    if constexpr (CM) {
 #pragma unroll
-    for (int i = 0; i < XT_HV / 4; ++i) {
-        const float4 q = reinterpret_cast<const float4 *>(p)[i];
-        v[4 * i] = q.x;
-        v[4 * i + 1] = q.y;
-        v[4 * i + 2] = q.z;
-        v[4 * i + 3] = q.w;
+        for (int i = 0; i < XT_HV; ++i) v[i] = p[i * cs];
+    } else {
+#pragma unroll
+        for (int i = 0; i < XT_HV / 4; ++i) {
+            const float4 q = reinterpret_cast<const float4 *>(p)[i];
+            v[4 * i] = q.x;
+            v[4 * i + 1] = q.y;
+            v[4 * i + 2] = q.z;
+            v[4 * i + 3] = q.w;
+        }
     }
 }
 
-__device__ __forceinline__ void st_half(float *p, const float (&v)[XT_HV])
+template <bool CM>
+__device__ __forceinline__ void st_half(float *p, size_t cs, const float (&v)[XT_HV])
 {
+    if constexpr (CM) {
 #pragma unroll
-    for (int i = 0; i < XT_HV / 4; ++i)
-        reinterpret_cast<float4 *>(p)[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+        for (int i = 0; i < XT_HV; ++i) p[i * cs] = v[i];
+    } else {
+#pragma unroll
+        for (int i = 0; i < XT_HV / 4; ++i)
+            reinterpret_cast<float4 *>(p)[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+    }
 }
 
 // XT_HV accumulator columns of this thread's lane, in two steps: tld_issue starts
@@ -163,7 +178,7 @@ __device__ __forceinline__ void tst(unsigned taddr, const float (&v)[XT_HV])
     tc::st16(taddr, v);
 }
 
-template <int N, int NP>
+template <int N, int NP, bool CM>
 __global__ void __launch_bounds__(XT_THREADS, 1) k_rows_tc(CurveDev c, int mode, StepArm arm)
 {
     using Cfg = XtCfg<N, NP>;
@@ -185,7 +200,12 @@ __global__ void __launch_bounds__(XT_THREADS, 1) k_rows_tc(CurveDev c, int mode,
     const bool issuer = warp == XT_PROD / 32;
     // producers: section row r (TMEM lane 32 (warp % 4) + lane), column half h of every chunk
     const int r = 32 * (warp & 3) + lane, h = (warp >> 2) & 1, co = h * XT_HV;
-    const int blk = blockIdx.x, nblk = gridDim.x;
+    const int blk = blockIdx.x, nblk = c.row_parts;
+    if (blk == nblk) {   // the extra CTA of the deferred form
+        pdl_wait();
+        finish_g2(c, XT_THREADS);
+        return;
+    }
     const int ns = c.ns, P = c.P;
     const int m = blk * XT_M + r;
     const bool has = !issuer && m < ns, in = has && m > 0 && m < P;
@@ -202,7 +222,7 @@ __global__ void __launch_bounds__(XT_THREADS, 1) k_rows_tc(CurveDev c, int mode,
     pdl_wait();
     const int g_done = arm.on ? 0 : sc->done;
     const long long g_step = sc->step, g_limit = arm.on ? g_step + arm.nsteps : sc->limit;
-    const double lamd = sc->lambda;
+    const double lamd = c.defer ? sc->lambda_next : sc->lambda;
     const long long wb = wait_bound(*sc);
     if (arm.on && blk == 0 && tid == 0) {
         sc->limit = g_limit;
@@ -213,6 +233,11 @@ __global__ void __launch_bounds__(XT_THREADS, 1) k_rows_tc(CurveDev c, int mode,
     if (mode == ROWS_STEP && (g_done || g_step >= g_limit)) {
         if (blk == 0 && tid == 0) sc->active = 0;
         return;
+    }
+    if (c.defer && blk == 0 && tid == 0) {
+        sc->active = 1;
+        sc->decided = 0;
+        sc->lambda = lamd;
     }
 
     if (warp == 0) {
@@ -302,7 +327,8 @@ __global__ void __launch_bounds__(XT_THREADS, 1) k_rows_tc(CurveDev c, int mode,
         // ---- producers: operand chunks, and the pointwise work between the products
         const unsigned lane_base = tmem + ((unsigned)(32 * (warp & 3)) << 16) + (unsigned)co;
         const float lam = (float)lamd;
-        const size_t ro = (size_t)(has ? m : 0) * N + co;
+        const size_t cs = CM ? (size_t)c.pitch : 1;   // words between two columns of a section
+        const size_t ro = CM ? (size_t)co * cs + (has ? m : 0) : (size_t)(has ? m : 0) * N + co;
         const float *Urow = U + ro, *Drow = D + ro;
         float *Rrow = R + ro, *Arow = A + ro;
         auto fail = [&]() {
@@ -355,9 +381,9 @@ __global__ void __launch_bounds__(XT_THREADS, 1) k_rows_tc(CurveDev c, int mode,
             tc::fence_after();
         };
         auto fetch_row = [&](const float *row) {
-            return [row, has = has](int cch, unsigned (&b)[XT_HV]) {
+            return [row, cs, has = has](int cch, unsigned (&b)[XT_HV]) {
                 float t[XT_HV];
-                if (has) ld_half(row + cch * XT_KC, t);
+                if (has) ld_half<CM>(row + cch * XT_KC * cs, cs, t);
                 else {
 #pragma unroll
                     for (int i = 0; i < XT_HV; ++i) t[i] = 0.f;
@@ -413,7 +439,7 @@ __global__ void __launch_bounds__(XT_THREADS, 1) k_rows_tc(CurveDev c, int mode,
                     s[3] += cw * (ur * ur + ui * ui);
                     s[4] += cw * (fr * fr + fi * fi);
                 }
-                if (has) st_half(Rrow + cch * XT_KC, rv);
+                if (has) st_half<CM>(Rrow + cch * XT_KC * cs, cs, rv);
             };
             unsigned u0[XT_HV], d0[XT_HV], w0[XT_HV], u1[XT_HV], d1[XT_HV], w1[XT_HV];
             fu(0, u0);
@@ -497,7 +523,7 @@ __global__ void __launch_bounds__(XT_THREADS, 1) k_rows_tc(CurveDev c, int mode,
                     ph[2 * i] = av.x;
                     ph[2 * i + 1] = av.y;
                 }
-                if (has) st_half(Arow + cch * XT_KC, ph);
+                if (has) st_half<CM>(Arow + cch * XT_KC * cs, cs, ph);
             };
             unsigned r0[XT_HV], p0[XT_HV], r1[XT_HV], p1[XT_HV];
             fr(0, r0);
@@ -560,6 +586,7 @@ __global__ void __launch_bounds__(XT_THREADS, 1) k_rows_tc(CurveDev c, int mode,
         c.bpart[(size_t)blk * 5 + tid] = tt;
     }
     // ---- last CTA: the FP64 reduction over the CTAs' partial sums
+    if (c.defer && mode == ROWS_STEP) return;   // the contraction sums the partials
     if (!last_cta_arrive(&sc->cnt_rows, (unsigned)nblk, am_last)) return;
     rows_finish<XT_THREADS>(c, mode, nblk, true, arm);
 }
@@ -595,14 +622,14 @@ __global__ void k_setup_xdft(CurveDev c)
     }
 }
 
-template <int N, int NP>
+template <int N, int NP, bool CM>
 cudaError_t rows_tc_run(const CurveDev &c, int mode, cudaStream_t st, StepArm arm)
 {
     using Cfg = XtCfg<N, NP>;
-    cudaError_t e = set_smem(k_rows_tc<N, NP>, Cfg::SMEM);
+    cudaError_t e = set_smem(k_rows_tc<N, NP, CM>, Cfg::SMEM);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3((c.ns + XT_M - 1) / XT_M);
+    cfg.gridDim = dim3(c.row_parts + c.defer);
     cfg.blockDim = dim3(XT_THREADS);
     cfg.dynamicSmemBytes = Cfg::SMEM;
     cfg.stream = st;
@@ -611,7 +638,7 @@ cudaError_t rows_tc_run(const CurveDev &c, int mode, cudaStream_t st, StepArm ar
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    e = cudaLaunchKernelEx(&cfg, k_rows_tc<N, NP>, c, mode, arm);
+    e = cudaLaunchKernelEx(&cfg, k_rows_tc<N, NP, CM>, c, mode, arm);
     if (e != cudaSuccess) return e;
     return cudaGetLastError();
 }
@@ -632,15 +659,21 @@ cudaError_t launch_setup_xdft(const CurveDev &c, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t launch_rows_tc(const CurveDev &c, int mode, cudaStream_t st, StepArm arm)
+template <bool CM>
+static cudaError_t rows_tc_dispatch(const CurveDev &c, int mode, cudaStream_t st, StepArm arm)
 {
     const bool three = c.xtc == 3;
     switch (c.nx) {
-    case 64: return three ? rows_tc_run<64, 3>(c, mode, st, arm) : rows_tc_run<64, 2>(c, mode, st, arm);
-    case 128: return three ? rows_tc_run<128, 3>(c, mode, st, arm) : rows_tc_run<128, 2>(c, mode, st, arm);
-    case 256: return three ? rows_tc_run<256, 3>(c, mode, st, arm) : rows_tc_run<256, 2>(c, mode, st, arm);
+    case 64: return three ? rows_tc_run<64, 3, CM>(c, mode, st, arm) : rows_tc_run<64, 2, CM>(c, mode, st, arm);
+    case 128: return three ? rows_tc_run<128, 3, CM>(c, mode, st, arm) : rows_tc_run<128, 2, CM>(c, mode, st, arm);
+    case 256: return three ? rows_tc_run<256, 3, CM>(c, mode, st, arm) : rows_tc_run<256, 2, CM>(c, mode, st, arm);
     default: return cudaErrorInvalidValue;
     }
+}
+
+cudaError_t launch_rows_tc(const CurveDev &c, int mode, cudaStream_t st, StepArm arm)
+{
+    return c.cc ? rows_tc_dispatch<true>(c, mode, st, arm) : rows_tc_dispatch<false>(c, mode, st, arm);
 }
 
 }  // namespace ks
