@@ -67,7 +67,7 @@ void header_sizes(int nb, const ks_params *p, size_t *cv_bytes, size_t *items_by
         tiles += (size_t)((p[i].ns + ks::DT_BM - 1) / ks::DT_BM) * ((p[i].nx + 31) / 32);
         modes += p[i].nx;   // column pairs, or the column form's columns
         if (p[i].scheme == KS_SCHEME_IMPLICIT)   // the increment's products (<= 2 per tile) and finishing pass (<= 8)
-            imp += 2 * (size_t)((p[i].nx + 63) / 64) * ((p[i].ns - 1) / 2 / 128 + 1) + 8;
+            imp += 2 * (size_t)((p[i].nx + 31) / 32) * ((p[i].ns - 1) / 2 / 32 + 1) + 8;
     }
     *cv_bytes = al256((size_t)nb * sizeof(ks::CurveDev));
     *items_bytes = al256(rows * sizeof(int2)) + al256(tiles * sizeof(int4)) + al256(modes * sizeof(int2)) +

@@ -338,29 +338,41 @@ ks_status setup_implicit(const CurveDev &c, cudaStream_t st)
 //   k_imp_back:   partial products of V_p with Y_p;
 //   k_imp_finish: the sum of the back partials in split order, unfolded into
 //                 U's update, and the step's bookkeeping in the last CTA.
-// The products are register-tiled on the CUDA cores: 128 x 64 outputs per CTA,
-// 8 x 4 per thread, K in steps of 16 through shared memory.
-constexpr int IM_BM = 128, IM_BN = 64, IM_BK = 16, IM_THREADS = 256, IM_TM = 8, IM_TN = 4;
+// The products are register-tiled on the CUDA cores, K in steps of 16 through shared
+// memory.  FP32: 128 x 64 outputs per CTA, 8 x 4 per thread.  FP64: 32 x 32 per CTA,
+// 4 x 2 per thread: the FP64 pipes (2 FMAs a cycle and SM) bound the product whatever
+// the tile, so it is cut fine enough to reach every SM (128 x 64 tiles put the paper's
+// M = 550, N = 64 on 24 of 152: 190 us a product, 32 x 32 on 144).
+constexpr int IM_THREADS = 256;   // of the elementwise passes
+template <typename T>
+struct ImCfg {
+    static constexpr int BM = sizeof(T) == 8 ? 32 : 128, BN = sizeof(T) == 8 ? 32 : 64, BK = 16, TM = sizeof(T) == 8 ? 4 : 8,
+                         TN = sizeof(T) == 8 ? 2 : 4, TX = BN / TN, NT = TX * (BM / TM);
+};
 
 template <typename T>
 struct ImSmem {
-    __align__(16) T As[IM_BK][IM_BM];
-    __align__(16) T Bs[IM_BK][IM_BN + 4];   // (B tiles of column-major operands are written k-fastest)
+    using C = ImCfg<T>;
+    __align__(16) T As[C::BK][C::BM];
+    __align__(16) T Bs[C::BK][C::BN + 4];   // (B tiles of column-major operands are written k-fastest)
 };
 
-// acc[i][l] += sum_{k in [kb, ke)} A[r0 + 8 ty + i][k] B(k, c0 + 4 tx + l);
+// acc[i][l] += sum_{k in [kb, ke)} A[r0 + TM ty + i][k] B(k, c0 + TN tx + l);
 // A row-major (nrows x lda), B(k, col) from `loadb` (called for k < ke, col < ncols),
 // contiguous in k (kfast) or in col.
 template <typename T, typename LoadB>
 __device__ __forceinline__ void im_tile(ImSmem<T> &sm, const T *A, int nrows, int lda, int r0, int kb, int ke, int c0,
-                                        int ncols, bool kfast, LoadB loadb, T (&acc)[IM_TM][IM_TN])
+                                        int ncols, bool kfast, LoadB loadb, T (&acc)[ImCfg<T>::TM][ImCfg<T>::TN])
 {
-    constexpr int AL = IM_BM * IM_BK / IM_THREADS, BL = IM_BK * IM_BN / IM_THREADS;
-    const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
-    const int ar = tid >> 1, ak = (tid & 1) * AL;   // A: a row and 8 consecutive k per thread
+    using C = ImCfg<T>;
+    constexpr int IM_BM = C::BM, IM_BN = C::BN, IM_BK = C::BK, IM_TM = C::TM, IM_TN = C::TN, NT = C::NT;
+    constexpr int AL = IM_BM * IM_BK / NT, BL = IM_BK * IM_BN / NT;
+    const int tid = threadIdx.x, tx = tid % C::TX, ty = tid / C::TX;
+    constexpr int KPT = IM_BK / AL;   // threads of a row of A: AL consecutive k each
+    const int ar = tid / KPT, ak = (tid % KPT) * AL;
     T ra[AL], rb[BL];
-    auto bk = [&](int q) { const int e = tid + q * IM_THREADS; return kfast ? e % IM_BK : e / IM_BN; };
-    auto bc = [&](int q) { const int e = tid + q * IM_THREADS; return kfast ? e / IM_BK : e % IM_BN; };
+    auto bk = [&](int q) { const int e = tid + q * NT; return kfast ? e % IM_BK : e / IM_BN; };
+    auto bc = [&](int q) { const int e = tid + q * NT; return kfast ? e / IM_BK : e % IM_BN; };
     auto fetch = [&](int k0) {
         const bool rok = r0 + ar < nrows;
         const T *arow = A + (size_t)(r0 + ar) * lda;
@@ -404,7 +416,7 @@ __device__ __forceinline__ void im_tile(ImSmem<T> &sm, const T *A, int nrows, in
 __device__ __forceinline__ void im_chunk(int n, int splits, int s, int &kb, int &ke)
 {
     int kc = (n + splits - 1) / splits;
-    kc = (kc + IM_BK - 1) / IM_BK * IM_BK;
+    kc = (kc + 15) / 16 * 16;
     kb = min(n, s * kc);
     ke = min(n, kb + kc);
 }
@@ -414,21 +426,22 @@ __device__ __forceinline__ void im_chunk(int n, int splits, int s, int &kb, int 
 template <typename T>
 __device__ __forceinline__ void imp_fwd_body(ImSmem<T> &sm, const CurveDev &c, int bx, int by, int bz, int splits)
 {
+    using C = ImCfg<T>;
     DevScalars *sc = c.sc;
     const int p = bz / splits, sp = bz % splits;
     const int M = c.ns - 2, h = M / 2, N = c.nx, ne = c.ine, np = p ? c.ino : ne;
-    const int r0 = by * IM_BM, c0 = bx * IM_BN;
+    const int r0 = by * C::BM, c0 = bx * C::BN;
     if (r0 >= np) return;
     int kb, ke;
     im_chunk(np, splits, sp, kb, ke);
     const T *G = (const T *)c.G;
     const T r2 = T(0.70710678118654752440);
     const T *A = (const T *)c.ivi + (p ? (size_t)ne * ne : 0);
-    T acc[IM_TM][IM_TN];
+    T acc[C::TM][C::TN];
 #pragma unroll
-    for (int i = 0; i < IM_TM; ++i)
+    for (int i = 0; i < C::TM; ++i)
 #pragma unroll
-        for (int l = 0; l < IM_TN; ++l) acc[i][l] = T(0);
+        for (int l = 0; l < C::TN; ++l) acc[i][l] = T(0);
     const size_t ms = c.ms, cs = c.cs;
     if (p == 0)
         im_tile<T>(sm, A, np, np, r0, kb, ke, c0, N, ms == 1, [&](int k, int col) -> T {
@@ -443,15 +456,15 @@ __device__ __forceinline__ void imp_fwd_body(ImSmem<T> &sm, const CurveDev &c, i
     const T lam = (T)sc->lambda, dtau = (T)sc->dtau, tl = T(2.0 * M_PI / c.L);
     const double *mu = c.imu + (p ? ne : 0);
     T *out = (T *)c.isc + (size_t)sp * M * N + (p ? (size_t)ne * c.ims : 0);
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const int tx = threadIdx.x % C::TX, ty = threadIdx.x / C::TX;
 #pragma unroll
-    for (int i = 0; i < IM_TM; ++i) {
-        const int r = r0 + IM_TM * ty + i;
+    for (int i = 0; i < C::TM; ++i) {
+        const int r = r0 + C::TM * ty + i;
         if (r >= np) continue;
         const T lm = lam * lam * (T)mu[r];
 #pragma unroll
-        for (int l = 0; l < IM_TN; ++l) {
-            const int col = c0 + IM_TN * tx + l;
+        for (int l = 0; l < C::TN; ++l) {
+            const int col = c0 + C::TN * tx + l;
             if (col >= N) continue;
             const T kw = tl * (T)(col >> 1), a = kw * kw * kw * kw - kw * kw;
             out[(size_t)r * c.ims + (size_t)col * c.ics] = dtau / (T(1) + dtau * (a * a - lm)) * acc[i][l];
@@ -465,20 +478,21 @@ template <typename T>
 __device__ __forceinline__ void imp_back_body(ImSmem<T> &sm, const CurveDev &c, int bx, int by, int bz, int splits_f,
                                               int splits)
 {
+    using C = ImCfg<T>;
     const int p = bz / splits, sp = bz % splits;
     const int M = c.ns - 2, N = c.nx, ne = c.ine, np = p ? c.ino : ne;
-    const int r0 = by * IM_BM, c0 = bx * IM_BN;
+    const int r0 = by * C::BM, c0 = bx * C::BN;
     if (r0 >= np) return;
     int kb, ke;
     im_chunk(np, splits, sp, kb, ke);
     const size_t off = p ? (size_t)ne * c.ims : 0, stride = (size_t)M * N;
     const T *Pf = (const T *)c.isc;
     const T *A = (const T *)c.iv + (p ? (size_t)ne * ne : 0);
-    T acc[IM_TM][IM_TN];
+    T acc[C::TM][C::TN];
 #pragma unroll
-    for (int i = 0; i < IM_TM; ++i)
+    for (int i = 0; i < C::TM; ++i)
 #pragma unroll
-        for (int l = 0; l < IM_TN; ++l) acc[i][l] = T(0);
+        for (int l = 0; l < C::TN; ++l) acc[i][l] = T(0);
     im_tile<T>(sm, A, np, np, r0, kb, ke, c0, N, c.ims == 1, [&](int k, int col) -> T {
         const T *y = Pf + off + (size_t)k * c.ims + (size_t)col * c.ics;
         T t = y[0];
@@ -486,14 +500,14 @@ __device__ __forceinline__ void imp_back_body(ImSmem<T> &sm, const CurveDev &c, 
         return t;
     }, acc);
     T *out = (T *)c.isc + (size_t)(c.isplits + sp) * stride + off;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+    const int tx = threadIdx.x % C::TX, ty = threadIdx.x / C::TX;
 #pragma unroll
-    for (int i = 0; i < IM_TM; ++i) {
-        const int r = r0 + IM_TM * ty + i;
+    for (int i = 0; i < C::TM; ++i) {
+        const int r = r0 + C::TM * ty + i;
         if (r >= np) continue;
 #pragma unroll
-        for (int l = 0; l < IM_TN; ++l) {
-            const int col = c0 + IM_TN * tx + l;
+        for (int l = 0; l < C::TN; ++l) {
+            const int col = c0 + C::TN * tx + l;
             if (col < N) out[(size_t)r * c.ims + (size_t)col * c.ics] = acc[i][l];
         }
     }
@@ -555,7 +569,7 @@ __global__ void __launch_bounds__(IM_THREADS) k_imp_sum(CurveDev c, int splits, 
 }
 
 template <typename T>
-__global__ void __launch_bounds__(IM_THREADS) k_imp_fwd(CurveDev c, int splits, int gate)
+__global__ void __launch_bounds__(ImCfg<T>::NT) k_imp_fwd(CurveDev c, int splits, int gate)
 {
     __shared__ ImSmem<T> sm;
     pdl_wait();
@@ -564,7 +578,7 @@ __global__ void __launch_bounds__(IM_THREADS) k_imp_fwd(CurveDev c, int splits, 
 }
 
 template <typename T>
-__global__ void __launch_bounds__(IM_THREADS) k_imp_back(CurveDev c, int splits, int gate)
+__global__ void __launch_bounds__(ImCfg<T>::NT) k_imp_back(CurveDev c, int splits, int gate)
 {
     __shared__ ImSmem<T> sm;
     pdl_wait();
@@ -584,7 +598,7 @@ __global__ void __launch_bounds__(IM_THREADS) k_imp_finish(CurveDev c, int split
 // Batched curves (one K chunk each): items (curve, bx, by, parity) of the two
 // products, (curve, bx, nbx, 0) of the finishing pass.
 template <typename T>
-__global__ void __launch_bounds__(IM_THREADS) k_imp_fwd_batch(const CurveDev *cv, const int4 *items)
+__global__ void __launch_bounds__(ImCfg<T>::NT) k_imp_fwd_batch(const CurveDev *cv, const int4 *items)
 {
     __shared__ ImSmem<T> sm;
     pdl_wait();
@@ -595,7 +609,7 @@ __global__ void __launch_bounds__(IM_THREADS) k_imp_fwd_batch(const CurveDev *cv
 }
 
 template <typename T>
-__global__ void __launch_bounds__(IM_THREADS) k_imp_back_batch(const CurveDev *cv, const int4 *items)
+__global__ void __launch_bounds__(ImCfg<T>::NT) k_imp_back_batch(const CurveDev *cv, const int4 *items)
 {
     __shared__ ImSmem<T> sm;
     pdl_wait();
@@ -617,11 +631,11 @@ __global__ void __launch_bounds__(IM_THREADS) k_imp_finish_batch(const CurveDev 
 }
 
 template <typename K, typename... Args>
-static cudaError_t imp_launch(K kern, dim3 grid, cudaStream_t st, Args... args)
+static cudaError_t imp_launch_n(K kern, dim3 grid, int block, cudaStream_t st, Args... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
-    cfg.blockDim = dim3(IM_THREADS);
+    cfg.blockDim = dim3(block);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -632,12 +646,20 @@ static cudaError_t imp_launch(K kern, dim3 grid, cudaStream_t st, Args... args)
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+template <typename K, typename... Args>
+static cudaError_t imp_launch(K kern, dim3 grid, cudaStream_t st, Args... args)
+{
+    return imp_launch_n(kern, grid, IM_THREADS, st, args...);
+}
+
 // K splits that bring the product's grid to about two CTAs per SM.
+template <typename T>
 static int imp_splits(const CurveDev &c)
 {
-    const int tiles = ((c.nx + IM_BN - 1) / IM_BN) * ((c.ine + IM_BM - 1) / IM_BM) * 2;
+    using C = ImCfg<T>;
+    const int tiles = ((c.nx + C::BN - 1) / C::BN) * ((c.ine + C::BM - 1) / C::BM) * 2;
     int s = (2 * 152 + tiles - 1) / tiles;
-    const int smax = std::max(1, c.ino / (4 * IM_BK));   // chunks of at least 64
+    const int smax = std::max(1, c.ino / (4 * C::BK));   // chunks of at least 64
     return std::max(1, std::min(std::min(s, c.isplits), smax));
 }
 
@@ -648,10 +670,11 @@ size_t implicit_scratch_bytes(int ns, int nx, int prec, int splits)
 
 void implicit_batch_items(const CurveDev &c, int curve, std::vector<int4> &prod, std::vector<int4> &fin)
 {
-    const int gx = (c.nx + IM_BN - 1) / IM_BN, gy = (c.ine + IM_BM - 1) / IM_BM;
+    const int bm = c.prec ? ImCfg<float>::BM : ImCfg<double>::BM, bn = c.prec ? ImCfg<float>::BN : ImCfg<double>::BN;
+    const int gx = (c.nx + bn - 1) / bn, gy = (c.ine + bm - 1) / bm;
     for (int p = 0; p < 2; ++p)
         for (int by = 0; by < gy; ++by) {
-            if (by * IM_BM >= (p ? c.ino : c.ine)) continue;
+            if (by * bm >= (p ? c.ino : c.ine)) continue;
             for (int bx = 0; bx < gx; ++bx) prod.push_back(make_int4(curve, bx, by, p));
         }
     const long total = (long)c.ine * c.nx;
@@ -680,14 +703,15 @@ template <typename T>
 static cudaError_t implicit_t(const CurveDev &c, int gate, cudaStream_t st)
 {
     if (sizeof(T) == 4 && c.ivtc) return implicit_tc_run(c, gate, st);
-    const int sp = imp_splits(c);
-    const int gx = (c.nx + IM_BN - 1) / IM_BN, gy = (c.ine + IM_BM - 1) / IM_BM;
-    cudaError_t e = imp_launch(k_imp_fwd<T>, dim3(gx, gy, 2 * sp), st, c, sp, gate);
+    using C = ImCfg<T>;
+    const int sp = imp_splits<T>(c);
+    const int gx = (c.nx + C::BN - 1) / C::BN, gy = (c.ine + C::BM - 1) / C::BM;
+    cudaError_t e = imp_launch_n(k_imp_fwd<T>, dim3(gx, gy, 2 * sp), C::NT, st, c, sp, gate);
     const long total = (long)c.ine * c.nx;
     if (e == cudaSuccess && sp > 1)
         e = imp_launch(k_imp_sum<T>, dim3((int)std::min<long>(4 * 152, (2 * total + IM_THREADS - 1) / IM_THREADS)), st,
                        c, sp, gate);
-    if (e == cudaSuccess) e = imp_launch(k_imp_back<T>, dim3(gx, gy, 2 * sp), st, c, sp, gate);
+    if (e == cudaSuccess) e = imp_launch_n(k_imp_back<T>, dim3(gx, gy, 2 * sp), C::NT, st, c, sp, gate);
     if (e != cudaSuccess) return e;
     const int gf = (int)std::min<long>(4 * 152, (total + IM_THREADS - 1) / IM_THREADS);
     return imp_launch(k_imp_finish<T>, dim3(gf), st, c, sp, gate);
@@ -705,12 +729,12 @@ cudaError_t launch_implicit_batch(int prec, const CurveDev *cv, const int4 *prod
     if (nprod <= 0) return cudaSuccess;
     cudaError_t e;
     if (prec) {
-        e = imp_launch(k_imp_fwd_batch<float>, dim3(nprod), st, cv, prod);
-        if (e == cudaSuccess) e = imp_launch(k_imp_back_batch<float>, dim3(nprod), st, cv, prod);
+        e = imp_launch_n(k_imp_fwd_batch<float>, dim3(nprod), ImCfg<float>::NT, st, cv, prod);
+        if (e == cudaSuccess) e = imp_launch_n(k_imp_back_batch<float>, dim3(nprod), ImCfg<float>::NT, st, cv, prod);
         if (e == cudaSuccess) e = imp_launch(k_imp_finish_batch<float>, dim3(nfin), st, cv, fin);
     } else {
-        e = imp_launch(k_imp_fwd_batch<double>, dim3(nprod), st, cv, prod);
-        if (e == cudaSuccess) e = imp_launch(k_imp_back_batch<double>, dim3(nprod), st, cv, prod);
+        e = imp_launch_n(k_imp_fwd_batch<double>, dim3(nprod), ImCfg<double>::NT, st, cv, prod);
+        if (e == cudaSuccess) e = imp_launch_n(k_imp_back_batch<double>, dim3(nprod), ImCfg<double>::NT, st, cv, prod);
         if (e == cudaSuccess) e = imp_launch(k_imp_finish_batch<double>, dim3(nfin), st, cv, fin);
     }
     return e;
