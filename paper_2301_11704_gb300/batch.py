@@ -83,7 +83,9 @@ class KSBatch:
         s = self.specs[i]
         out = torch.empty((s.Ns, s.N), dtype=self.dtype, device=self.device)
         check(self.lib.ks_batch_get_state(self.handle, int(i), out.data_ptr()))
-        self.stream.synchronize()
+        # on torch's current stream the tensor's readers are ordered after the copy
+        if self.stream != torch.cuda.current_stream(self.device):
+            self.stream.synchronize()
         return out
 
     def autotune(self, steps: int = 8) -> dict:

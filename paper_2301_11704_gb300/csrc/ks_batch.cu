@@ -41,6 +41,7 @@ struct ks_batch {
     ks::CurveDev *cv_dev = nullptr;
     unsigned char *items_dev = nullptr; // item area
     size_t items_cap = 0;
+    unsigned char *stage_dev = nullptr; // staging area (Stage)
     std::vector<Group> rows, dts;
     std::vector<Group> ccs;             // (curve, column) items of the column form, one group per length
     std::vector<Group> ffts;            // (curve, mode) items of the FFT-form curves, one group per F
@@ -57,6 +58,30 @@ struct ks_batch {
 namespace {
 
 size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
+
+// Staging area of the batch's set-up and reads: what the per-curve copies of amplitudes,
+// fields and scalars would otherwise be is one copy each.
+struct Stage {
+    size_t init, gather, index, voff, amps, vp, total;   // offsets
+    Stage(int nb, const ks_params *p)
+    {
+        size_t fields = 0;
+        for (int i = 0; i < nb; ++i) fields += (size_t)ks::MAX_PERT * p[i].nx;
+        size_t o = 0;
+        auto take = [&o](size_t bytes) {
+            const size_t at = o;
+            o += al256(bytes);
+            return at;
+        };
+        init = take((size_t)nb * sizeof(ks::ScalarInit));
+        gather = take((size_t)nb * sizeof(ks::DevScalars));
+        index = take((size_t)nb * sizeof(int));
+        voff = take((size_t)nb * sizeof(int));
+        amps = take((size_t)nb * ks::MAX_PERT * sizeof(double));
+        vp = take(fields * sizeof(double));
+        total = o;
+    }
+};
 
 // Bytes of the batch header: curve array and the largest item lists.
 void header_sizes(int nb, const ks_params *p, size_t *cv_bytes, size_t *items_bytes)
@@ -285,11 +310,11 @@ ks_status enqueue(ks_batch *b, int64_t nsteps, double tol)
 ks_status read_all(ks_batch *b, std::vector<ks::DevScalars> &h)
 {
     h.resize(b->nb);
-    for (int i = 0; i < b->nb; ++i) {
-        cudaError_t e = cudaMemcpyAsync(&h[i], b->cv[i].sc, sizeof(ks::DevScalars), cudaMemcpyDeviceToHost, b->st);
-        if (e != cudaSuccess) return ks::report_error(KS_ECUDA, "scalar read: %s", cudaGetErrorString(e));
-    }
-    cudaError_t e = cudaStreamSynchronize(b->st);
+    ks::DevScalars *g = (ks::DevScalars *)(b->stage_dev + Stage(b->nb, b->p.data()).gather);
+    cudaError_t e = ks::launch_scalars_gather(b->cv_dev, g, b->nb, b->st);
+    if (e == cudaSuccess)
+        e = cudaMemcpyAsync(h.data(), g, (size_t)b->nb * sizeof(ks::DevScalars), cudaMemcpyDeviceToHost, b->st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->st);
     if (e != cudaSuccess) return ks::report_error(KS_ECUDA, "scalar read: %s", cudaGetErrorString(e));
     for (size_t i = 0; i < h.size(); ++i)
         if (h[i].err)
@@ -303,6 +328,78 @@ ks_status eval_all(ks_batch *b)
     for (const Group &g : b->rows)
         if (e == cudaSuccess) e = launch_rows_group(b, g, ks::ROWS_EVAL, b->st);
     if (e != cudaSuccess) return ks::report_error(KS_ECUDA, "batched evaluation: %s", cudaGetErrorString(e));
+    return KS_OK;
+}
+
+// Trial curves of every curve with npert perturbation modes, D_t u of them and the
+// scalars reset: the column-form curves together (one launch per N and per length),
+// the others one by one.  The host arrays may go once the stream is synchronised.
+ks_status init_all(ks_batch *b, int npert, const double *amps_host, const double *vp_host, std::vector<int> &voff)
+{
+    const Stage sg(b->nb, b->p.data());
+    voff.resize(b->nb);
+    size_t nv = 0;
+    for (int i = 0; i < b->nb; ++i) {
+        voff[i] = (int)nv;
+        nv += (size_t)npert * b->cv[i].nx;
+    }
+    double *amps = (double *)(b->stage_dev + sg.amps), *vp = (double *)(b->stage_dev + sg.vp);
+    int *vo = (int *)(b->stage_dev + sg.voff);
+    cudaError_t e = cudaSuccess;
+    if (npert > 0) {
+        e = cudaMemcpyAsync(amps, amps_host, (size_t)b->nb * npert * 8, cudaMemcpyHostToDevice, b->st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(vp, vp_host, nv * 8, cudaMemcpyHostToDevice, b->st);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(vo, voff.data(), b->nb * sizeof(int), cudaMemcpyHostToDevice, b->st);
+    }
+    for (const Group &g : b->rows)
+        if (e == cudaSuccess && g.key >= CM_KEY)
+            e = ks::launch_trial_batch_cm(b->prec, g.key - CM_KEY, 2 * b->row_warps, b->cv_dev,
+                                          (const int2 *)(b->items_dev + g.off), g.count, npert, amps, vp, vo, b->st);
+    for (const Group &g : b->ccs)
+        if (e == cudaSuccess)
+            e = ks::launch_cc_batch(b->prec, g.key, b->cv_dev, (const int2 *)(b->items_dev + g.off), g.count, ks::GM_STORE,
+                                    0, 0, b->st);
+    for (int i = 0; i < b->nb && e == cudaSuccess; ++i) {
+        const ks::CurveDev &c = b->cv[i];
+        if (c.cc) continue;
+        if (npert > 0) {
+            e = cudaMemcpyAsync(c.pert + c.nx, amps + (size_t)i * npert, npert * 8, cudaMemcpyDeviceToDevice, b->st);
+            if (e == cudaSuccess)
+                e = cudaMemcpyAsync(c.pert + c.nx + ks::MAX_PERT, vp + voff[i], (size_t)npert * c.nx * 8,
+                                    cudaMemcpyDeviceToDevice, b->st);
+        }
+        if (e == cudaSuccess) e = ks::launch_trial(c, 0.0, 0, npert, b->st);
+        if (e == cudaSuccess) e = ks::launch_row_fwd_x(c, c.U, 0, b->st);
+        if (e == cudaSuccess) e = ks::launch_dt(c, ks::GM_STORE, 0, 0, b->st);
+    }
+    if (e == cudaSuccess)
+        e = ks::launch_scalars_init_batch(b->cv_dev, (const ks::ScalarInit *)(b->stage_dev + sg.init), b->nb, b->st);
+    if (e != cudaSuccess) return ks::report_error(KS_ECUDA, "trial curves: %s", cudaGetErrorString(e));
+    return KS_OK;
+}
+
+// Set-up of the column form's tables, the batch's curves together.
+ks_status setup_columns(ks_batch *b)
+{
+    std::map<int, std::vector<int>> by_len;
+    int ns_max = 0;
+    for (int i = 0; i < b->nb; ++i) {
+        if (!b->cv[i].cc) continue;
+        by_len[b->cv[i].cc].push_back(i);
+        ns_max = std::max(ns_max, b->cv[i].ns);
+    }
+    if (by_len.empty()) return KS_OK;
+    cudaError_t e = ks::launch_setup_cc_tables(b->prec, b->cv_dev, b->nb, ns_max, b->st);
+    int *index = (int *)(b->stage_dev + Stage(b->nb, b->p.data()).index);
+    size_t at = 0;
+    for (auto &kv : by_len) {
+        const int n = (int)kv.second.size();
+        if (e == cudaSuccess) e = cudaMemcpyAsync(index + at, kv.second.data(), n * sizeof(int), cudaMemcpyHostToDevice, b->st);
+        if (e == cudaSuccess) e = ks::launch_setup_cc_spectra(b->prec, kv.first, b->cv_dev, index + at, n, b->st);
+        at += n;
+    }
+    if (e == cudaSuccess) e = cudaStreamSynchronize(b->st);   // host vectors die at return
+    if (e != cudaSuccess) return ks::report_error(KS_ECUDA, "batch set-up: %s", cudaGetErrorString(e));
     return KS_OK;
 }
 
@@ -352,7 +449,7 @@ size_t ks_batch_workspace_bytes(int32_t nb, const ks_params *params)
     if (validate_batch(nb, params) != KS_OK) return 0;
     size_t cvb, itb;
     header_sizes(nb, params, &cvb, &itb);
-    size_t total = cvb + itb;
+    size_t total = cvb + itb + Stage(nb, params).total;
     for (int i = 0; i < nb; ++i)
         total += ks::make_layout(params[i].ns, params[i].nx, ks::storage32(params[i].precision), 0, 0,
                                  params[i].s_transform, 0, 0, params[i].scheme == KS_SCHEME_IMPLICIT,
@@ -387,7 +484,8 @@ ks_status ks_batch_create(int32_t nb, const ks_params *params, const double *u_p
     b->cv_dev = (ks::CurveDev *)base;
     b->items_dev = base + cvb;
     b->items_cap = itb;
-    size_t o = cvb + itb;
+    b->stage_dev = base + cvb + itb;
+    size_t o = cvb + itb + Stage(nb, params).total;
     b->cv.resize(nb);
     size_t xoff = 0;
     for (int i = 0; i < nb; ++i) {
@@ -408,17 +506,21 @@ ks_status ks_batch_create(int32_t nb, const ks_params *params, const double *u_p
         if (e == cudaSuccess)
             e = cudaMemsetAsync(c.pert, 0, (size_t)(c.nx + ks::MAX_PERT + ks::MAX_PERT * c.nx) * 8, b->st);
         if (e == cudaSuccess) e = ks::launch_setup(c, params[i].dtau, b->st);
-        if (e == cudaSuccess)
-            e = ks::launch_scalars_init(c, params[i].lambda, params[i].lambda_free, params[i].dtau,
-                                        params[i].dtau_lambda, params[i].conv, b->st);
-        if (e == cudaSuccess) e = ks::launch_trial(c, 0.0, 0, 0, b->st);
-        if (e == cudaSuccess) e = ks::launch_row_fwd_x(c, c.U, 0, b->st);
-        if (e == cudaSuccess) e = ks::launch_dt(c, ks::GM_STORE, 0, 0, b->st);
         if (e != cudaSuccess) s = ks::report_error(KS_ECUDA, "batch set-up of curve %d: %s", i, cudaGetErrorString(e));
         xoff += c.nx;
     }
-    if (s == KS_OK && b->impl) s = setup_implicit_all(b);
+    std::vector<ks::ScalarInit> init(nb);
+    for (int i = 0; i < nb; ++i)
+        init[i] = {params[i].lambda, params[i].dtau, params[i].dtau_lambda, params[i].lambda_free, params[i].conv};
+    if (s == KS_OK && cudaMemcpyAsync(b->stage_dev + Stage(nb, params).init, init.data(), nb * sizeof(init[0]),
+                                      cudaMemcpyHostToDevice, b->st) != cudaSuccess)
+        s = ks::report_error(KS_ECUDA, "batch set-up: copy of the scalars");
+    std::vector<int> voff;
     if (s == KS_OK) s = build_items(b);
+    if (s == KS_OK) s = setup_columns(b);
+    if (s == KS_OK) s = init_all(b, 0, nullptr, nullptr, voff);
+    if (s == KS_OK && b->impl) s = setup_implicit_all(b);
+    if (s == KS_OK && cudaStreamSynchronize(b->st) != cudaSuccess) s = ks::report_error(KS_ECUDA, "batch set-up");
     if (s != KS_OK) {
         delete b;
         return s;
@@ -432,25 +534,9 @@ ks_status ks_batch_init_trial(ks_batch *b, int32_t npert, const double *amps_hos
     if (!b) return ks::report_error(KS_EINVAL, "batch handle is NULL");
     if (npert < 0 || npert > ks::MAX_PERT) return ks::report_error(KS_EINVAL, "npert must be in [0, %d]", ks::MAX_PERT);
     if (npert > 0 && (!amps_host || !vp_host)) return ks::report_error(KS_EINVAL, "amps_host and vp_host are required");
-    size_t voff = 0;
-    for (int i = 0; i < b->nb; ++i) {
-        const ks::CurveDev &c = b->cv[i];
-        const ks_params &p = b->p[i];
-        cudaError_t e = cudaSuccess;
-        if (npert > 0) {
-            e = cudaMemcpyAsync(c.pert + c.nx, amps_host + (size_t)i * npert, npert * 8, cudaMemcpyHostToDevice, b->st);
-            if (e == cudaSuccess)
-                e = cudaMemcpyAsync(c.pert + c.nx + ks::MAX_PERT, vp_host + voff, (size_t)npert * c.nx * 8,
-                                    cudaMemcpyHostToDevice, b->st);
-        }
-        if (e == cudaSuccess) e = ks::launch_trial(c, 0.0, 0, npert, b->st);
-        if (e == cudaSuccess) e = ks::launch_row_fwd_x(c, c.U, 0, b->st);
-        if (e == cudaSuccess) e = ks::launch_dt(c, ks::GM_STORE, 0, 0, b->st);
-        if (e == cudaSuccess)
-            e = ks::launch_scalars_init(c, p.lambda, p.lambda_free, p.dtau, p.dtau_lambda, p.conv, b->st);
-        if (e != cudaSuccess) return ks::report_error(KS_ECUDA, "trial curve %d: %s", i, cudaGetErrorString(e));
-        voff += (size_t)npert * c.nx;
-    }
+    std::vector<int> voff;
+    const ks_status s = init_all(b, npert, amps_host, vp_host, voff);
+    if (s != KS_OK) return s;
     cudaError_t e = cudaStreamSynchronize(b->st);
     if (e != cudaSuccess) return ks::report_error(KS_ECUDA, "trial curves: %s", cudaGetErrorString(e));
     return KS_OK;

@@ -718,9 +718,21 @@ __global__ void k_cc_finish(const __grid_constant__ CurveDev c)
 // up to a constant that follows from sum_{l<2P} g[l] = kappa_0 = P / pi; g[1 - l] = g[l].
 // First the increments and the other tables (row scales -sin^2(theta) / S and, for
 // FP32 storage, the quadrature weights in it), then the sum by one CTA.
+// Set-up kernels run over curves: one (by value), or the batch's (blockIdx.y).
+struct CurveSet {
+    CurveDev one;
+    const CurveDev *many;   // with `index`: the curves of one length
+    const int *index;
+    __device__ const CurveDev &get() const { return many ? many[index ? index[blockIdx.y] : blockIdx.y] : one; }
+    CurveSet from(int o) const { return {one, many && !index ? many + o : many, index ? index + o : index}; }
+};
+constexpr int GRID_Y = 32768;   // curves per launch
+
 template <typename T>
-__global__ void __launch_bounds__(256) k_cc_tables(CurveDev c)
+__global__ void __launch_bounds__(256) k_cc_tables(const __grid_constant__ CurveSet cs)
 {
+    const CurveDev &c = cs.get();
+    if (!c.cc) return;
     const int P = c.P;
     double *g = (double *)c.X;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < c.ns; i += gridDim.x * blockDim.x) {
@@ -734,8 +746,10 @@ __global__ void __launch_bounds__(256) k_cc_tables(CurveDev c)
     }
 }
 
-__global__ void __launch_bounds__(1024) k_cc_kernel(CurveDev c)
+__global__ void __launch_bounds__(1024) k_cc_kernel(const __grid_constant__ CurveSet cs)
 {
+    const CurveDev &c = cs.get();
+    if (!c.cc) return;
     __shared__ double wpre[32], wtot[32];
     const int P = c.P, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int ch = (P + 1023) / 1024, q0 = 1 + tid * ch, q1 = min(P + 1, q0 + ch);
@@ -773,8 +787,9 @@ __global__ void __launch_bounds__(1024) k_cc_kernel(CurveDev c)
     }
 }
 
-__global__ void __launch_bounds__(256) k_cc_specA(CurveDev c, int L, int A)
+__global__ void __launch_bounds__(256) k_cc_specA(const __grid_constant__ CurveSet cs, int L, int A)
 {
+    const CurveDev &c = cs.get();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double2 *wA = (double2 *)smem_raw;   // e^(-2 pi i p / 4A), p < 4A
     for (int p = threadIdx.x; p < 4 * A; p += blockDim.x) {
@@ -810,8 +825,9 @@ __global__ void __launch_bounds__(256) k_cc_specA(CurveDev c, int L, int A)
 }
 
 template <class F, int CS>
-__global__ void __launch_bounds__(256) k_cc_specB(CurveDev c, int A)
+__global__ void __launch_bounds__(256) k_cc_specB(const __grid_constant__ CurveSet cs, int A)
 {
+    const CurveDev &c = cs.get();
     using T = typename F::type;
     constexpr int L = F::L * CS;   // CS classes of F::L frequencies
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -863,25 +879,45 @@ cudaError_t cc_launch(void (*kern)(KArgs...), int grid, int block, size_t smem, 
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-template <class F, int CS>
-cudaError_t setup_run(const CurveDev &c, cudaStream_t st)
+template <typename T>
+cudaError_t setup_tables(const CurveSet &cs, int n, int ns_max, cudaStream_t st)
 {
-    using T = typename F::type;
+    for (int o = 0; o < n; o += GRID_Y) {
+        const CurveSet part = cs.from(o);
+        const int k = n - o < GRID_Y ? n - o : GRID_Y;
+        k_cc_tables<T><<<dim3((ns_max + 255) / 256, k), 256, 0, st>>>(part);
+        k_cc_kernel<<<dim3(1, k), 1024, 0, st>>>(part);
+    }
+    return cudaGetLastError();
+}
+
+template <class F, int CS>
+cudaError_t setup_spectra(const CurveSet &cs, int nc, cudaStream_t st)
+{
     constexpr int L = F::L * CS;
     int A = 1;
     while (A * A < L) A <<= 1;
     const int B = L / A, n = 2 * L > F::TW * CS ? 2 * L : F::TW * CS;
-    k_cc_tables<T><<<(c.ns + 255) / 256, 256, 0, st>>>(c);
-    k_cc_kernel<<<1, 1024, 0, st>>>(c);
-    k_cc_specA<<<(2 * L + 255) / 256, 256, (size_t)4 * A * sizeof(double2), st>>>(c, L, A);
-    k_cc_specB<F, CS><<<(n + 255) / 256, 256, (size_t)B * sizeof(double2), st>>>(c, A);
+    for (int o = 0; o < nc; o += GRID_Y) {
+        const CurveSet part = cs.from(o);
+        const int k = nc - o < GRID_Y ? nc - o : GRID_Y;
+        k_cc_specA<<<dim3((2 * L + 255) / 256, k), 256, (size_t)4 * A * sizeof(double2), st>>>(part, L, A);
+        k_cc_specB<F, CS><<<dim3((n + 255) / 256, k), 256, (size_t)B * sizeof(double2), st>>>(part, A);
+    }
     return cudaGetLastError();
 }
 
 template <typename T>
 cudaError_t setup_t(const CurveDev &c, cudaStream_t st)
 {
-    return cc_dispatch<T>(c.cc, [&](auto f) { return setup_run<decltype(f), 1>(c, st); }, cudaErrorInvalidValue);
+    const CurveSet cs = {c, nullptr, nullptr};
+    cudaError_t e = setup_tables<T>(cs, 1, c.ns, st);
+    if (e != cudaSuccess) return e;
+    if (c.ccl > 1)
+        return cx_dispatch(
+            c.cc, c.ccl, [&](auto f, auto k) { return setup_spectra<decltype(f), decltype(k)::value>(cs, 1, st); },
+            cudaErrorInvalidValue);
+    return cc_dispatch<T>(c.cc, [&](auto f) { return setup_spectra<decltype(f), 1>(cs, 1, st); }, cudaErrorInvalidValue);
 }
 
 cudaError_t run_cx(const CurveDev &c, int mode, int discrete, int gate, cudaStream_t st)
@@ -963,11 +999,20 @@ int cc_warps(int L, int prec, int cs)
 
 cudaError_t launch_setup_cc(const CurveDev &c, cudaStream_t st)
 {
-    if (c.ccl > 1)
-        return cx_dispatch(
-            c.cc, c.ccl, [&](auto f, auto cs) { return setup_run<decltype(f), decltype(cs)::value>(c, st); },
-            cudaErrorInvalidValue);
     return c.prec ? setup_t<float>(c, st) : setup_t<double>(c, st);
+}
+
+cudaError_t launch_setup_cc_tables(int prec, const CurveDev *cv, int nb, int ns_max, cudaStream_t st)
+{
+    const CurveSet cs = {CurveDev{}, cv, nullptr};
+    return prec ? setup_tables<float>(cs, nb, ns_max, st) : setup_tables<double>(cs, nb, ns_max, st);
+}
+
+cudaError_t launch_setup_cc_spectra(int prec, int L, const CurveDev *cv, const int *index, int n, cudaStream_t st)
+{
+    const CurveSet cs = {CurveDev{}, cv, index};
+    auto run = [&](auto f) { return setup_spectra<decltype(f), 1>(cs, n, st); };
+    return prec ? cc_dispatch<float>(L, run, cudaErrorInvalidValue) : cc_dispatch<double>(L, run, cudaErrorInvalidValue);
 }
 
 cudaError_t launch_cc(const CurveDev &c, int mode, int discrete, int gate, cudaStream_t st)

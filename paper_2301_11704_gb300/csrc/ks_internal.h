@@ -319,6 +319,7 @@ struct CurveDev {
     // summed beside the next row phase (or by launch_cc_finish); lambda_next is the
     // current lambda from the contraction on.
     int defer, row_parts, g2_parts;
+    int batched;              // a curve of a batch
     int ims, ics;             // the same of the implicit step's partials (rows of M, columns of N)
     void *cctw, *ccs;         // twiddles; spectra (T_k, H_k) / L, L pairs of complex values
     void *ccr;                // row scales -sin^2(theta_j) / S
@@ -434,6 +435,10 @@ inline int f4b_splits(int F, int prec, int (&F1s)[3])
 size_t cc_twiddles(int L, int prec, int cs);
 int cc_warps(int L, int prec, int cs);   // of a column's CTAs
 cudaError_t launch_setup_cc(const CurveDev &c, cudaStream_t st);
+// Set-up of a batch's column-form curves: the tables of every curve, then the spectra of
+// the curves of one length (n of them, index: their places in cv).
+cudaError_t launch_setup_cc_tables(int prec, const CurveDev *cv, int nb, int ns_max, cudaStream_t st);
+cudaError_t launch_setup_cc_spectra(int prec, int L, const CurveDev *cv, const int *index, int n, cudaStream_t st);
 cudaError_t launch_cc(const CurveDev &c, int mode, int discrete, int gate, cudaStream_t st);
 // Deferred form: the |G|^2 of the last update and its lambda, for calls that end with an update.
 cudaError_t launch_cc_finish(const CurveDev &c, cudaStream_t st);
@@ -445,6 +450,9 @@ int cm_sections(int nx, int ns, int prec, int want, int single);
 cudaError_t launch_rows_cm(const CurveDev &c, int mode, cudaStream_t st, StepArm arm);
 cudaError_t launch_rows_cm_batch(int prec, int N, int sec, const CurveDev *cv, const int2 *items, int nitems, int mode,
                                  cudaStream_t st);
+// Trial curves of a batch into the spectral state, over the row phase's items.
+cudaError_t launch_trial_batch_cm(int prec, int N, int sec, const CurveDev *cv, const int2 *items, int nitems, int npert,
+                                  const double *amps, const double *vp, const int *voff, cudaStream_t st);
 cudaError_t launch_row_fwd_x_cm(const CurveDev &c, void *spec, cudaStream_t st);
 cudaError_t launch_row_fwd_cm(const CurveDev &c, const void *phys, void *spec, cudaStream_t st);
 cudaError_t launch_row_inv_cm(const CurveDev &c, const void *spec, void *phys, int scale_mode, cudaStream_t st);
@@ -492,6 +500,14 @@ cudaError_t launch_rows_batch(int prec, int N, int warps, const CurveDev *cv, co
                               cudaStream_t st);
 cudaError_t launch_dt_batch(int prec, int bn, const CurveDev *cv, const int4 *items, int nitems, int mode,
                             int discrete, int gate, cudaStream_t st);
+// Scalars of a batch: reset (launch_scalars_init of every curve; lambda: nb values), and
+// gathered into one array.
+struct ScalarInit {
+    double lambda, dtau, dtau_lambda;
+    int lambda_free, conv;
+};
+cudaError_t launch_scalars_init_batch(const CurveDev *cv, const ScalarInit *init, int nb, cudaStream_t st);
+cudaError_t launch_scalars_gather(const CurveDev *cv, DevScalars *out, int nb, cudaStream_t st);
 cudaError_t launch_set_limit_batch(const CurveDev *cv, int nb, long long nsteps, double tol, cudaStream_t st);
 // FFT-form s-contraction over (curve, mode) items; smem sized for F_max
 cudaError_t launch_sconv_batch(int prec, int F_max, const CurveDev *cv, const int2 *items, int nitems, int mode,

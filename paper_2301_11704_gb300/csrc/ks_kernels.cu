@@ -225,6 +225,7 @@ CurveDev bind_layout(const ks_params *p, const Layout &l, void *base)
     d.pitch = l.pitch;
     d.rsec = l.rsec;
     d.defer = l.cc && !l.impl && l.single;
+    d.batched = !l.single;
     d.g2_parts = l.cc ? l.w * cc_warps(l.cc, d.prec, l.ccl) : 0;
     d.ccl = l.ccl;
     d.row_parts = l.xtc ? (p->ns + 127) / 128 : l.row_blocks;
@@ -350,6 +351,29 @@ __global__ void k_scalars_init(DevScalars *sc, unsigned *tcnt, int ntiles, doubl
         z.limit = 0;
         *sc = z;
     }
+}
+
+__global__ void k_scalars_init_batch(const CurveDev *cv, const ScalarInit *init)
+{
+    const CurveDev &c = cv[blockIdx.x];
+    for (int i = threadIdx.x; i < c.tiles_r * c.tiles_c; i += blockDim.x) c.tcnt[i] = 0u;
+    if (threadIdx.x == 0) {
+        const ScalarInit &p = init[blockIdx.x];
+        DevScalars z{};
+        z.lambda = p.lambda;
+        z.lambda_next = p.lambda;
+        z.lambda_free = p.lambda_free;
+        z.dtau = p.dtau;
+        z.dtau_lambda = p.dtau_lambda;
+        z.conv = p.conv;
+        *c.sc = z;
+    }
+}
+
+__global__ void k_scalars_gather(const CurveDev *cv, DevScalars *out, int nb)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < nb) out[i] = *cv[i].sc;
 }
 
 __global__ void k_set_wait_cycles(DevScalars *sc, long long cycles)
@@ -1194,7 +1218,7 @@ cudaError_t launch_setup(const CurveDev &c, double dtau, cudaStream_t st)
     else k_setup<double><<<grid, 256, 0, st>>>(c, dtau);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess && c.xtc) e = launch_setup_xdft(c, st);
-    if (e == cudaSuccess && c.cc) return launch_setup_cc(c, st);
+    if (e == cudaSuccess && c.cc) return c.batched ? e : launch_setup_cc(c, st);   // (a batch's curves together)
     if (e != cudaSuccess || c.F == 0) return e;
     if (c.f4) return launch_setup_f4(c, st);
     const int g2 = (c.F + 255) / 256;
@@ -1214,6 +1238,18 @@ cudaError_t launch_scalars_init(const CurveDev &c, double lambda, int lambda_fre
 {
     k_scalars_init<<<1, 256, 0, st>>>(c.sc, c.tcnt, c.tiles_r * c.tiles_c, lambda, lambda_free, dtau, dtau_lambda,
                                       conv);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_scalars_init_batch(const CurveDev *cv, const ScalarInit *init, int nb, cudaStream_t st)
+{
+    k_scalars_init_batch<<<nb, 64, 0, st>>>(cv, init);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_scalars_gather(const CurveDev *cv, DevScalars *out, int nb, cudaStream_t st)
+{
+    k_scalars_gather<<<(nb + 63) / 64, 64, 0, st>>>(cv, out, nb);
     return cudaGetLastError();
 }
 

@@ -465,6 +465,74 @@ __global__ void __launch_bounds__(CmCfg<Tc, To, N, SEC>::NTHR) k_row_fwd_cm(cons
     CmTile<To, N, SEC, C::NTHR>::store(tile, spec, c.pitch, c.W, c.hs, m0);
 }
 
+// Trial curves (eq. KSE_initial_curve with a = 0, plus the perturbation) of a batch's
+// column-form curves straight into the spectral state, in FP64: work item (curve, row
+// block) per CTA.  The sections' factors (tanh and the sines) are formed once per
+// section.  amps: npert per curve; vp: the curves' [npert][N] fields, curve i's at voff[i].
+template <typename To, int N, int SEC>
+__global__ void __launch_bounds__(CmCfg<double, To, N, SEC>::NTHR)
+    k_trial_batch_cm(const CurveDev *cv, const int2 *items, int npert, const double *amps, const double *vp, const int *voff)
+{
+    using C = CmCfg<double, To, N, SEC>;
+    using F = typename C::F;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double fac[SEC][2 + MAX_PERT];
+    cpx<double> *tw = C::tw(smem_raw);
+    To *tile = C::tile(smem_raw, 0);
+    const int2 it = items[blockIdx.x];
+    const CurveDev &c = cv[it.x];
+    const int tid = threadIdx.x, pr = tid / C::LPS, t = tid % C::LPS, m0 = it.y * SEC, ns = c.ns, P = c.P;
+    const int sa = 2 * pr;
+    cpx<double> *buf = C::buf(smem_raw) + (size_t)pr * C::BUFS;
+    auto sync = [] { __syncwarp(); };
+    row_twiddles<F, N, C::NTHR>(tw, [&](int k) { return row_root<double>(c, k); });
+    for (int e = tid; e < SEC * (1 + npert); e += C::NTHR) {
+        const int s = e / (1 + npert), q = e % (1 + npert), m = m0 + s;
+        if (q == 0) {
+            double sn, co, h = m == 0 ? 1.0 : -1.0;
+            if (m > 0 && m < P) {
+                sincospi((double)m / (double)P, &sn, &co);
+                h = tanh(c.s0 + c.S * co / sn);
+            }
+            fac[s][0] = m < ns ? 0.5 * (1.0 + h) : 0.0;
+            fac[s][1] = m < ns ? 0.5 * (1.0 - h) : 0.0;
+        } else {
+            double sn = 0.0, co;
+            if (m > 0 && m < P) sincospi((double)(((long long)q * m) % (2LL * P)) / (double)P, &sn, &co);
+            fac[s][1 + q] = amps[(size_t)it.x * npert + q - 1] * sn;
+        }
+    }
+    __syncthreads();
+    const double *up = c.ends, *um = c.ends + N, *v0 = vp + voff[it.x];
+    cpx<double> v[F::E];
+#pragma unroll
+    for (int e = 0; e < F::E; ++e) {   // the grid index in the digit order dit() starts from
+        const int n = F::freq(t, e);
+        const double a = up[n], b = um[n];
+        v[e] = {fac[sa][0] * a + fac[sa][1] * b, fac[sa + 1][0] * a + fac[sa + 1][1] * b};
+        for (int p = 0; p < npert; ++p) {
+            const double x = v0[p * N + n];
+            v[e].x += fac[sa][2 + p] * x;
+            v[e].y += fac[sa + 1][2 + p] * x;
+        }
+    }
+    F::template dit<false>(v, buf, tw, t, sync);
+    F::template store<0>(v, buf, t);
+    sync();
+#pragma unroll
+    for (int i = 0; i < C::HE; ++i) {
+        const int j = t + C::LPS * i;
+        cpx<double> A, B;
+        unpack_pair<F, N>(buf, j, A, B);
+        A = project(A, j, c.sym);
+        B = project(B, j, c.sym);
+        *reinterpret_cast<cpx<To> *>(tile + sa * C::TS + 2 * j) = {(To)A.x, (To)A.y};
+        *reinterpret_cast<cpx<To> *>(tile + (sa + 1) * C::TS + 2 * j) = {(To)B.x, (To)B.y};
+    }
+    __syncthreads();
+    CmTile<To, N, SEC, C::NTHR>::store(tile, (To *)c.U, c.pitch, c.W, c.hs, m0);
+}
+
 template <typename T, int N, int SEC>
 __global__ void __launch_bounds__(CmCfg<T, T, N, SEC>::NTHR) k_row_inv_cm(const __grid_constant__ CurveDev c, const T *spec,
                                                                           T *phys, int scale_mode)
@@ -621,6 +689,26 @@ cudaError_t launch_rows_cm_batch(int prec, int N, int sec, const CurveDev *cv, c
     if (nitems <= 0) return cudaSuccess;
     return prec ? rows_batch_t<float>(N, sec, cv, items, nitems, mode, st)
                 : rows_batch_t<double>(N, sec, cv, items, nitems, mode, st);
+}
+
+template <typename T>
+static cudaError_t trial_batch_t(int N_, int sec, const CurveDev *cv, const int2 *items, int nitems, int npert,
+                                 const double *amps, const double *vp, const int *voff, cudaStream_t st)
+{
+    return cm_dispatch<T>(N_, sec, [&](auto nn, auto ss) {
+        constexpr int N = decltype(nn)::value, SEC = decltype(ss)::value;
+        using C = CmCfg<double, T, N, SEC>;
+        return cm_launch(k_trial_batch_cm<T, N, SEC>, nitems, C::NTHR, C::bytes(1), st, false, cv, items, npert, amps, vp,
+                         voff);
+    });
+}
+
+cudaError_t launch_trial_batch_cm(int prec, int N, int sec, const CurveDev *cv, const int2 *items, int nitems, int npert,
+                                  const double *amps, const double *vp, const int *voff, cudaStream_t st)
+{
+    if (nitems <= 0) return cudaSuccess;
+    return prec ? trial_batch_t<float>(N, sec, cv, items, nitems, npert, amps, vp, voff, st)
+                : trial_batch_t<double>(N, sec, cv, items, nitems, npert, amps, vp, voff, st);
 }
 
 cudaError_t launch_row_fwd_x_cm(const CurveDev &c, void *spec, cudaStream_t st)
