@@ -474,6 +474,8 @@ ks_status ks_batch_create(int32_t nb, const ks_params *params, const double *u_p
     b->nb = nb;
     b->prec = ks::storage32(params[0].precision);
     b->discrete = params[0].adjoint == KS_ADJ_DISCRETE;
+    // FP32: 16 sections per row CTA (64-byte runs of a column; 6% of the 256-curve step)
+    if (b->prec) b->row_warps = 2 * ks::ROWS_WARPS;
     b->impl = params[0].scheme == KS_SCHEME_IMPLICIT;
     b->st = (cudaStream_t)stream;
     cudaGetDevice(&b->device);

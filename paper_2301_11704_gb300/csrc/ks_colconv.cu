@@ -45,26 +45,31 @@ namespace ks {
 
 namespace {
 
-// The transform of each length.  FP32: 16 values per thread (8 up to L = 512), 32
-// from L = 8192 on (two exchanges instead of three); FP64: 8 (the FP64 pipe needs
-// warps more than it needs fewer exchanges).
-template <typename T, int L>
-struct CcPlan;
-template <> struct CcPlan<float, 128> { using F = RegFft<float, 128, 4, true, false, 4, 4, 4, 2>; };
-template <> struct CcPlan<float, 256> { using F = RegFft<float, 256, 8, true, false, 8, 8, 4>; };
-template <> struct CcPlan<float, 512> { using F = RegFft<float, 512, 8, true, false, 8, 8, 8>; };
-template <> struct CcPlan<float, 1024> { using F = RegFft<float, 1024, 16, true, false, 16, 16, 4>; };
-template <> struct CcPlan<float, 2048> { using F = RegFft<float, 2048, 16, true, false, 16, 16, 8>; };
-template <> struct CcPlan<float, 4096> { using F = RegFft<float, 4096, 16, true, false, 16, 16, 16>; };
-template <> struct CcPlan<float, 8192> { using F = RegFft<float, 8192, 32, true, false, 32, 32, 8>; };
-template <> struct CcPlan<float, 16384> { using F = RegFft<float, 16384, 32, true, false, 32, 32, 16>; };
-template <> struct CcPlan<double, 128> { using F = RegFft<double, 128, 4, true, true, 4, 4, 4, 2>; };
-template <> struct CcPlan<double, 256> { using F = RegFft<double, 256, 8, true, true, 8, 8, 4>; };
-template <> struct CcPlan<double, 512> { using F = RegFft<double, 512, 8, true, true, 8, 8, 8>; };
-template <> struct CcPlan<double, 1024> { using F = RegFft<double, 1024, 8, true, true, 8, 8, 4, 4>; };
-template <> struct CcPlan<double, 2048> { using F = RegFft<double, 2048, 8, true, true, 8, 8, 8, 4>; };
-template <> struct CcPlan<double, 4096> { using F = RegFft<double, 4096, 8, true, true, 8, 8, 8, 8>; };
-template <> struct CcPlan<double, 8192> { using F = RegFft<double, 8192, 16, true, true, 16, 16, 8, 4>; };
+// The transform of each length (B: of batched curves).  FP32: 16 values per thread, 32
+// from L = 8192 on (two exchanges instead of three: 35.7 against 43.6 us a step's
+// contraction at 256 x 8000), 8 up to L = 512 and for single curves up to 2048, which
+// are bound by the latency of a column's chain (L = 1024: 10.7 against 12.9 us; the
+// 256-curve batch, bound by throughput, takes 0.74 ms a step with 8 and 0.57 with
+// 16).  FP64: few values, to give every quarter of an SM's FP64 pipes a warp.
+template <typename T, int L, bool B = false>
+struct CcPlan : CcPlan<T, L, false> {};
+template <> struct CcPlan<float, 128, false> { using F = RegFft<float, 128, 4, true, false, 4, 4, 4, 2>; };
+template <> struct CcPlan<float, 256, false> { using F = RegFft<float, 256, 8, true, false, 8, 8, 4>; };
+template <> struct CcPlan<float, 512, false> { using F = RegFft<float, 512, 8, true, false, 8, 8, 8>; };
+template <> struct CcPlan<float, 1024, false> { using F = RegFft<float, 1024, 8, true, false, 8, 8, 4, 4>; };
+template <> struct CcPlan<float, 1024, true> { using F = RegFft<float, 1024, 16, true, false, 16, 16, 4>; };
+template <> struct CcPlan<float, 2048, false> { using F = RegFft<float, 2048, 8, true, false, 8, 8, 8, 4>; };
+template <> struct CcPlan<float, 2048, true> { using F = RegFft<float, 2048, 16, true, false, 16, 16, 8>; };
+template <> struct CcPlan<float, 4096, false> { using F = RegFft<float, 4096, 16, true, false, 16, 16, 16>; };
+template <> struct CcPlan<float, 8192, false> { using F = RegFft<float, 8192, 32, true, false, 32, 32, 8>; };
+template <> struct CcPlan<float, 16384, false> { using F = RegFft<float, 16384, 32, true, false, 32, 32, 16>; };
+template <> struct CcPlan<double, 128, false> { using F = RegFft<double, 128, 2, true, true, 2, 2, 2, 2, 2, 2, 2>; };
+template <> struct CcPlan<double, 256, false> { using F = RegFft<double, 256, 2, true, true, 2, 2, 2, 2, 2, 2, 2, 2>; };
+template <> struct CcPlan<double, 512, false> { using F = RegFft<double, 512, 4, true, true, 4, 4, 4, 4, 2>; };
+template <> struct CcPlan<double, 1024, false> { using F = RegFft<double, 1024, 8, true, true, 8, 8, 4, 4>; };
+template <> struct CcPlan<double, 2048, false> { using F = RegFft<double, 2048, 8, true, true, 8, 8, 8, 4>; };
+template <> struct CcPlan<double, 4096, false> { using F = RegFft<double, 4096, 8, true, true, 8, 8, 8, 8>; };
+template <> struct CcPlan<double, 8192, false> { using F = RegFft<double, 8192, 16, true, true, 16, 16, 8, 4>; };
 
 // The split form (a column over a cluster of CS CTAs): the transform of one class of
 // L / CS frequencies.  A warp's FP64 instruction takes about 64 cycles on its quarter
@@ -94,19 +99,19 @@ auto cx_dispatch(int L, int cs, Fn &&fn, decltype(fn(typename CxPlan<256>::F(), 
     return none;
 }
 
-template <typename T, typename Fn>
-auto cc_dispatch(int L, Fn &&fn, decltype(fn(typename CcPlan<T, 128>::F())) none)
+template <typename T, bool B, typename Fn>
+auto cc_dispatch(int L, Fn &&fn, decltype(fn(typename CcPlan<T, 128, B>::F())) none)
 {
     switch (L) {
-    case 128: return fn(typename CcPlan<T, 128>::F());
-    case 256: return fn(typename CcPlan<T, 256>::F());
-    case 512: return fn(typename CcPlan<T, 512>::F());
-    case 1024: return fn(typename CcPlan<T, 1024>::F());
-    case 2048: return fn(typename CcPlan<T, 2048>::F());
-    case 4096: return fn(typename CcPlan<T, 4096>::F());
-    case 8192: return fn(typename CcPlan<T, 8192>::F());
+    case 128: return fn(typename CcPlan<T, 128, B>::F());
+    case 256: return fn(typename CcPlan<T, 256, B>::F());
+    case 512: return fn(typename CcPlan<T, 512, B>::F());
+    case 1024: return fn(typename CcPlan<T, 1024, B>::F());
+    case 2048: return fn(typename CcPlan<T, 2048, B>::F());
+    case 4096: return fn(typename CcPlan<T, 4096, B>::F());
+    case 8192: return fn(typename CcPlan<T, 8192, B>::F());
     case 16384:
-        if constexpr (sizeof(T) == 4) return fn(typename CcPlan<T, 16384>::F());
+        if constexpr (sizeof(T) == 4) return fn(typename CcPlan<T, 16384, B>::F());
         break;
     default: break;
     }
@@ -917,7 +922,7 @@ cudaError_t setup_t(const CurveDev &c, cudaStream_t st)
         return cx_dispatch(
             c.cc, c.ccl, [&](auto f, auto k) { return setup_spectra<decltype(f), decltype(k)::value>(cs, 1, st); },
             cudaErrorInvalidValue);
-    return cc_dispatch<T>(c.cc, [&](auto f) { return setup_spectra<decltype(f), 1>(cs, 1, st); }, cudaErrorInvalidValue);
+    return cc_dispatch<T, false>(c.cc, [&](auto f) { return setup_spectra<decltype(f), 1>(cs, 1, st); }, cudaErrorInvalidValue);
 }
 
 cudaError_t run_cx(const CurveDev &c, int mode, int discrete, int gate, cudaStream_t st)
@@ -953,7 +958,7 @@ cudaError_t run_cx(const CurveDev &c, int mode, int discrete, int gate, cudaStre
 template <typename T>
 cudaError_t run_t(const CurveDev &c, int mode, int discrete, int gate, cudaStream_t st)
 {
-    return cc_dispatch<T>(
+    return cc_dispatch<T, false>(
         c.cc,
         [&](auto f) {
             using F = decltype(f);
@@ -970,7 +975,7 @@ template <typename T>
 cudaError_t batch_t(int L, const CurveDev *cv, const int2 *items, int nitems, int mode, int discrete, int gate,
                     cudaStream_t st)
 {
-    return cc_dispatch<T>(
+    return cc_dispatch<T, true>(
         L,
         [&](auto f) {
             using F = decltype(f);
@@ -983,18 +988,19 @@ cudaError_t batch_t(int L, const CurveDev *cv, const int2 *items, int nitems, in
 
 }  // namespace
 
-size_t cc_twiddles(int L, int prec, int cs)
+size_t cc_twiddles(int L, int prec, int cs, int batched)
 {
     if (cs > 1) return cx_dispatch(L, cs, [](auto f, auto) { return (size_t)decltype(f)::TW; }, (size_t)0) * cs;
     const auto n = [](auto f) { return (size_t)decltype(f)::TW; };
-    return prec ? cc_dispatch<float>(L, n, (size_t)0) : cc_dispatch<double>(L, n, (size_t)0);
+    if (batched) return prec ? cc_dispatch<float, true>(L, n, (size_t)0) : cc_dispatch<double, true>(L, n, (size_t)0);
+    return prec ? cc_dispatch<float, false>(L, n, (size_t)0) : cc_dispatch<double, false>(L, n, (size_t)0);
 }
 
 int cc_warps(int L, int prec, int cs)
 {
     if (cs > 1) return cx_dispatch(L, cs, [](auto f, auto) { return decltype(f)::NT / 32; }, 0) * cs;
     const auto n = [](auto f) { return decltype(f)::NT / 32; };
-    return prec ? cc_dispatch<float>(L, n, 0) : cc_dispatch<double>(L, n, 0);
+    return prec ? cc_dispatch<float, false>(L, n, 0) : cc_dispatch<double, false>(L, n, 0);
 }
 
 cudaError_t launch_setup_cc(const CurveDev &c, cudaStream_t st)
@@ -1012,7 +1018,7 @@ cudaError_t launch_setup_cc_spectra(int prec, int L, const CurveDev *cv, const i
 {
     const CurveSet cs = {CurveDev{}, cv, index};
     auto run = [&](auto f) { return setup_spectra<decltype(f), 1>(cs, n, st); };
-    return prec ? cc_dispatch<float>(L, run, cudaErrorInvalidValue) : cc_dispatch<double>(L, run, cudaErrorInvalidValue);
+    return prec ? cc_dispatch<float, true>(L, run, cudaErrorInvalidValue) : cc_dispatch<double, true>(L, run, cudaErrorInvalidValue);
 }
 
 cudaError_t launch_cc(const CurveDev &c, int mode, int discrete, int gate, cudaStream_t st)

@@ -432,7 +432,7 @@ inline int f4b_splits(int F, int prec, int (&F1s)[3])
 // Column form (ks_colconv.cu; c.cc set): twiddle entries of a length, set-up of its
 // tables, the s-contraction in the modes of launch_dt (GM_STEP: the update and
 // D_t u of the updated state), and over the (curve, column) items of a batch.
-size_t cc_twiddles(int L, int prec, int cs);
+size_t cc_twiddles(int L, int prec, int cs, int batched);
 int cc_warps(int L, int prec, int cs);   // of a column's CTAs
 cudaError_t launch_setup_cc(const CurveDev &c, cudaStream_t st);
 // Set-up of a batch's column-form curves: the tables of every curve, then the spectra of

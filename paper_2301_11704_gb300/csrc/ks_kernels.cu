@@ -160,7 +160,7 @@ Layout make_layout(int ns, int nx, int prec, int allow_split, int bn, int s_tran
     l.off_ends = off; off += al256((size_t)2 * nx * 8);
     l.off_pert = off; off += al256((size_t)(nx + MAX_PERT + MAX_PERT * nx) * 8);
     l.off_sc = off; off += al256(sizeof(DevScalars));
-    l.off_cctw = off; off += l.cc ? al256(cc_twiddles(l.cc, prec, l.ccl) * 2 * b) : 0;
+    l.off_cctw = off; off += l.cc ? al256(cc_twiddles(l.cc, prec, l.ccl, !allow_split) * 2 * b) : 0;
     l.off_ccs = off; off += l.cc ? al256((size_t)l.cc * 4 * b) : 0;
     l.off_ccr = off; off += l.cc ? al256((size_t)ns * b) : 0;
     l.off_ccx = off; off += l.cc ? al256((size_t)l.cc * 2 * 16) : 0;
