@@ -219,7 +219,8 @@ static cudaError_t launch_rows_group(const ks_batch *b, const Group &g, int mode
     const int2 *items = (const int2 *)(b->items_dev + g.off);
     if (g.key >= CM_KEY)
         return ks::launch_rows_cm_batch(b->prec, g.key - CM_KEY, 2 * b->row_warps, b->cv_dev, items, g.count, mode, st);
-    return ks::launch_rows_batch(b->prec, g.key, b->row_warps, b->cv_dev, items, g.count, mode, st);
+    return ks::launch_rows_batch(b->prec, g.key, b->row_warps, b->cv_dev, items, g.count,
+                                 mode == ks::ROWS_COST ? ks::ROWS_EVAL : mode, st);
 }
 
 ks_status launch_step(ks_batch *b, cudaStream_t st)
@@ -326,7 +327,7 @@ ks_status eval_all(ks_batch *b)
 {
     cudaError_t e = cudaSuccess;
     for (const Group &g : b->rows)
-        if (e == cudaSuccess) e = launch_rows_group(b, g, ks::ROWS_EVAL, b->st);
+        if (e == cudaSuccess) e = launch_rows_group(b, g, ks::ROWS_COST, b->st);
     if (e != cudaSuccess) return ks::report_error(KS_ECUDA, "batched evaluation: %s", cudaGetErrorString(e));
     return KS_OK;
 }

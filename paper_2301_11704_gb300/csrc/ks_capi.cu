@@ -479,7 +479,7 @@ ks_status ks_curve_cost(ks_curve *c, double *J2, double *J_arc)
     if (s != KS_OK) return s;
     DeviceGuard g(c->device);
     if (!g.ok) return fail(KS_ECUDA, "cannot select the curve's device");
-    KS_CUDA(ks::launch_rows(c->d, ks::ROWS_EVAL, c->st));
+    KS_CUDA(ks::launch_rows(c->d, ks::ROWS_COST, c->st));
     ks::DevScalars h;
     s = read_scalars(c, &h);
     if (s != KS_OK) return s;
@@ -534,7 +534,7 @@ ks_status ks_curve_descend(ks_curve *c, int64_t nsteps, double tol, int64_t *ste
     KS_CUDA(cudaMemcpyAsync(c->h0, c->d.sc, sizeof(ks::DevScalars), cudaMemcpyDeviceToHost, c->st));
     s = enqueue_steps(c, nsteps, tol);
     if (s != KS_OK) return s;
-    KS_CUDA(ks::launch_rows(c->d, ks::ROWS_EVAL, c->st));
+    KS_CUDA(ks::launch_rows(c->d, ks::ROWS_COST, c->st));
     ks::DevScalars h;
     s = read_scalars(c, &h);
     if (s != KS_OK) return s;
@@ -600,6 +600,10 @@ ks_status ks_curve_set_state(ks_curve *c, const void *u_dev, double lambda, doub
     // storage, double-float (the linear term of f multiplies each coefficient by
     // a_j ~ k_j^4: a coefficient must keep its own relative precision, not that
     // of the largest one, which an FP32 transform would give it)
+    if (c->d.cc) {
+        KS_CUDA(ks::launch_row_fwd_cm(c->d, u_dev, c->d.U, ks::SetScalars{lambda, tau, 1}, c->st));
+        return refresh_dt_u(c);
+    }
     KS_CUDA(ks::launch_row_fwd(c->d, u_dev, c->d.U, c->st));
     s = refresh_dt_u(c);
     if (s != KS_OK) return s;

@@ -392,6 +392,18 @@ __device__ __forceinline__ int rows_finish(const CurveDev &c, int mode, int nblk
     return go;
 }
 
+// A state given by the caller: lambda, tau, and the step counter restarted.
+__device__ __forceinline__ void set_scalars(DevScalars *sc, double lambda, double tau)
+{
+    sc->lambda = lambda;
+    sc->lambda_next = lambda;
+    sc->tau = tau;
+    sc->step = 0;
+    sc->limit = 0;
+    sc->done = 0;
+    sc->status = 0;
+}
+
 // Deferred form (CurveDev::defer): the sum of the last update's |G|^2 partials (one per
 // warp of each column, c.g2_parts) in a fixed order, in a CTA of its own (nt threads, at
 // most 256) beside the next row phase.

@@ -220,7 +220,9 @@ __host__ __device__ inline long long wait_bound(const DevScalars &s) { return s.
 // Gates of the kernels of one descent step:
 //   rows kernel:   skip when done or step >= limit (clears `active`)
 //   gemm kernels:  skip when !active
-enum RowsMode { ROWS_STEP = 0, ROWS_EVAL = 1 };
+// ROWS_COST: the evaluation's scalars alone (r^ and the adjoint are neither formed
+// further nor stored by the column-major row phases; the others run ROWS_EVAL).
+enum RowsMode { ROWS_STEP = 0, ROWS_EVAL = 1, ROWS_COST = 2 };
 // GM_STEP (clustered four-step form only): GM_UPDATE, then GM_STORE of the
 // updated state in the same launch.
 // The three-launch four-step form on the Toeplitz and Hankel parts (single
@@ -454,7 +456,12 @@ cudaError_t launch_rows_cm_batch(int prec, int N, int sec, const CurveDev *cv, c
 cudaError_t launch_trial_batch_cm(int prec, int N, int sec, const CurveDev *cv, const int2 *items, int nitems, int npert,
                                   const double *amps, const double *vp, const int *voff, cudaStream_t st);
 cudaError_t launch_row_fwd_x_cm(const CurveDev &c, void *spec, cudaStream_t st);
-cudaError_t launch_row_fwd_cm(const CurveDev &c, const void *phys, void *spec, cudaStream_t st);
+// with `set.on` also sets lambda and tau and resets the step counter (launch_set_lambda_tau)
+struct SetScalars {
+    double lambda, tau;
+    int on;
+};
+cudaError_t launch_row_fwd_cm(const CurveDev &c, const void *phys, void *spec, SetScalars set, cudaStream_t st);
 cudaError_t launch_row_inv_cm(const CurveDev &c, const void *spec, void *phys, int scale_mode, cudaStream_t st);
 
 // Split-BF16 tensor-core row phase (ks_rows_tc.cu; c.xtc set): bytes of its DFT

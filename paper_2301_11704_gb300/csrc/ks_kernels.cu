@@ -394,15 +394,7 @@ __global__ void k_set_limit(DevScalars *sc, long long nsteps, double tol)
 
 __global__ void k_set_lambda_tau(DevScalars *sc, double lambda, double tau)
 {
-    if (threadIdx.x == 0 && blockIdx.x == 0) {
-        sc->lambda = lambda;
-        sc->lambda_next = lambda;
-        sc->tau = tau;
-        sc->step = 0;
-        sc->limit = 0;
-        sc->done = 0;
-        sc->status = 0;
-    }
+    if (threadIdx.x == 0 && blockIdx.x == 0) set_scalars(sc, lambda, tau);
 }
 
 // Trial curve (eq. KSE_initial_curve) on the grid, physical, into X:
@@ -1307,7 +1299,7 @@ cudaError_t launch_row_fwd_x(const CurveDev &c, void *spec, int keep_ends, cudaS
 
 cudaError_t launch_row_fwd(const CurveDev &c, const void *phys, void *spec, cudaStream_t st)
 {
-    if (c.cc) return launch_row_fwd_cm(c, phys, spec, st);
+    if (c.cc) return launch_row_fwd_cm(c, phys, spec, SetScalars{0.0, 0.0, 0}, st);
     return c.prec ? row_fwd_t<float, dfloat, float>(c, phys, spec, 0, st)
                   : row_fwd_t<double, double, double>(c, phys, spec, 0, st);
 }
@@ -1322,6 +1314,7 @@ cudaError_t launch_rows(const CurveDev &c, int mode, cudaStream_t st, StepArm ar
 {
     if (c.xtc) return launch_rows_tc(c, mode, st, arm);
     if (c.cc) return launch_rows_cm(c, mode, st, arm);
+    if (mode == ROWS_COST) mode = ROWS_EVAL;
     return c.prec ? rows_t<float>(c, mode, st, arm) : rows_t<double>(c, mode, st, arm);
 }
 

@@ -77,7 +77,7 @@ extern "C" ks_status ks_cost_noalloc(const ks_params *p, const void *u_dev, doub
     if ((e = ks::launch_row_fwd_x(d, d.U, 0, st)) != cudaSuccess) return na_fail(KS_ECUDA, "forward transform", e);
     // D_t u, then the row phase with the FP64 cost reduction
     if ((e = ks::launch_dt(d, ks::GM_STORE, 0, 0, st)) != cudaSuccess) return na_fail(KS_ECUDA, "D_t u", e);
-    if ((e = ks::launch_rows(d, ks::ROWS_EVAL, st)) != cudaSuccess) return na_fail(KS_ECUDA, "row phase", e);
+    if ((e = ks::launch_rows(d, ks::ROWS_COST, st)) != cudaSuccess) return na_fail(KS_ECUDA, "row phase", e);
     k_export_cost<<<1, 32, 0, st>>>(d.sc, out_dev);
     if ((e = cudaGetLastError()) != cudaSuccess) return na_fail(KS_ECUDA, "export", e);
     return KS_OK;

@@ -282,6 +282,7 @@ __device__ __forceinline__ void rows_cm_body(const CurveDev &c, int mode, int bl
         *reinterpret_cast<cpx<T> *>(ua + 2 * j) = ra[i];
         *reinterpret_cast<cpx<T> *>(ub + 2 * j) = rb[i];
     }
+    if (mode != ROWS_COST) {
     sync();   // every partner value has been read
     // the packed spectrum of i k r^ -> r_x on the grid -> DFT of u r_x
 #pragma unroll
@@ -313,6 +314,7 @@ __device__ __forceinline__ void rows_cm_body(const CurveDev &c, int mode, int bl
         if (j == 0) oa.y = ob.y = T(0);
         *reinterpret_cast<cpx<T> *>(da + 2 * j) = oa;
         *reinterpret_cast<cpx<T> *>(db + 2 * j) = ob;
+    }
     }
     // per-section norms |q_m|^2 = L sum_j c_j |q^_j|^2.  The eight sums are halved at the
     // first butterfly levels (a lane keeps the half its bit selects, one addition per
@@ -369,8 +371,10 @@ __device__ __forceinline__ void rows_cm_body(const CurveDev &c, int mode, int bl
         }
     }
     __syncthreads();
-    CmTile<T, N, SEC, NTHR>::store(tu, as_global((T *)c.R), pitch, W, hs, m0);
-    CmTile<T, N, SEC, NTHR>::store(td, as_global((T *)c.A), pitch, W, hs, m0);
+    if (mode != ROWS_COST) {
+        CmTile<T, N, SEC, NTHR>::store(tu, as_global((T *)c.R), pitch, W, hs, m0);
+        CmTile<T, N, SEC, NTHR>::store(td, as_global((T *)c.A), pitch, W, hs, m0);
+    }
     if (tid < 32) {
         // the CTA's sums over its sections in FP64: value q in lanes 4 q .. 4 q + 3, a quarter
         // of the sections each (few FP64 instructions: each takes about 64 cycles)
@@ -429,7 +433,7 @@ __device__ __forceinline__ cpx<T> row_root(const CurveDev &c, int k)
 // to the storage type To.
 template <typename Ti, typename Tc, typename To, int N, int SEC>
 __global__ void __launch_bounds__(CmCfg<Tc, To, N, SEC>::NTHR) k_row_fwd_cm(const __grid_constant__ CurveDev c,
-                                                                            const Ti *phys, To *spec)
+                                                                            const Ti *phys, To *spec, SetScalars set)
 {
     using C = CmCfg<Tc, To, N, SEC>;
     using F = typename C::F;
@@ -441,6 +445,8 @@ __global__ void __launch_bounds__(CmCfg<Tc, To, N, SEC>::NTHR) k_row_fwd_cm(cons
     cpx<Tc> *buf = C::buf(smem_raw) + (size_t)pr * C::BUFS;
     auto sync = [] { __syncwarp(); };
     row_twiddles<F, N, C::NTHR>(tw, [&](int k) { return row_root<Tc>(c, k); });
+    pdl_wait();
+    if (set.on && blockIdx.x == 0 && tid == 0) set_scalars(c.sc, set.lambda, set.tau);
     cpx<Tc> v[F::E];
 #pragma unroll
     for (int e = 0; e < F::E; ++e) {   // the grid index in the digit order dit() starts from
@@ -547,8 +553,9 @@ __global__ void __launch_bounds__(CmCfg<T, T, N, SEC>::NTHR) k_row_inv_cm(const 
     cpx<T> *buf = C::buf(smem_raw) + (size_t)pr * C::BUFS;
     auto sync = [] { __syncwarp(); };
     CmTile<T, N, SEC, C::NTHR> x;
-    x.fetch(spec, c.pitch, c.W, m0);
     row_twiddles<F, N, C::NTHR>(tw, [&](int k) { return row_root<T>(c, k); });
+    pdl_wait();
+    x.fetch(spec, c.pitch, c.W, m0);
     x.put(tile, c.W, c.hs, m0, ns);
     T fa = 1, fb = 1;
     if (scale_mode == 1) {   // Euclidean gradient: -2 dx w_m, zero on the end rows
@@ -642,13 +649,13 @@ cudaError_t rows_batch_t(int N_, int sec, const CurveDev *cv, const int2 *items,
 }
 
 template <typename Ti, typename Tc, typename To>
-cudaError_t fwd_t(const CurveDev &c, const void *phys, void *spec, cudaStream_t st)
+cudaError_t fwd_t(const CurveDev &c, const void *phys, void *spec, SetScalars set, cudaStream_t st)
 {
     return cm_dispatch<float>(c.nx, 8, [&](auto nn, auto ss) {
         constexpr int N = decltype(nn)::value, SEC = decltype(ss)::value;
         using C = CmCfg<Tc, To, N, SEC>;
-        return cm_launch(k_row_fwd_cm<Ti, Tc, To, N, SEC>, (c.ns + SEC - 1) / SEC, C::NTHR, C::bytes(1), st, false, c,
-                         (const Ti *)phys, (To *)spec);
+        return cm_launch(k_row_fwd_cm<Ti, Tc, To, N, SEC>, (c.ns + SEC - 1) / SEC, C::NTHR, C::bytes(1), st, true, c,
+                         (const Ti *)phys, (To *)spec, set);
     });
 }
 
@@ -658,7 +665,7 @@ cudaError_t inv_t(const CurveDev &c, const void *spec, void *phys, int scale_mod
     return cm_dispatch<float>(c.nx, 8, [&](auto nn, auto ss) {
         constexpr int N = decltype(nn)::value, SEC = decltype(ss)::value;
         using C = CmCfg<T, T, N, SEC>;
-        return cm_launch(k_row_inv_cm<T, N, SEC>, (c.ns + SEC - 1) / SEC, C::NTHR, C::bytes(1), st, false, c,
+        return cm_launch(k_row_inv_cm<T, N, SEC>, (c.ns + SEC - 1) / SEC, C::NTHR, C::bytes(1), st, true, c,
                          (const T *)spec, (T *)phys, scale_mode);
     });
 }
@@ -713,12 +720,13 @@ cudaError_t launch_trial_batch_cm(int prec, int N, int sec, const CurveDev *cv, 
 
 cudaError_t launch_row_fwd_x_cm(const CurveDev &c, void *spec, cudaStream_t st)
 {
-    return c.prec ? fwd_t<double, double, float>(c, c.X, spec, st) : fwd_t<double, double, double>(c, c.X, spec, st);
+    const SetScalars none = {0.0, 0.0, 0};
+    return c.prec ? fwd_t<double, double, float>(c, c.X, spec, none, st) : fwd_t<double, double, double>(c, c.X, spec, none, st);
 }
 
-cudaError_t launch_row_fwd_cm(const CurveDev &c, const void *phys, void *spec, cudaStream_t st)
+cudaError_t launch_row_fwd_cm(const CurveDev &c, const void *phys, void *spec, SetScalars set, cudaStream_t st)
 {
-    return c.prec ? fwd_t<float, dfloat, float>(c, phys, spec, st) : fwd_t<double, double, double>(c, phys, spec, st);
+    return c.prec ? fwd_t<float, dfloat, float>(c, phys, spec, set, st) : fwd_t<double, double, double>(c, phys, spec, set, st);
 }
 
 cudaError_t launch_row_inv_cm(const CurveDev &c, const void *spec, void *phys, int scale_mode, cudaStream_t st)

@@ -262,6 +262,8 @@ __global__ void __launch_bounds__(XT_THREADS, 1) k_rows_tc(CurveDev c, int mode,
     volatile int *vbad = &sbad;
     float s[5] = {0.f, 0.f, 0.f, 0.f, 0.f};   // row sums |r|^2, |d|^2, <d,r>, |u|^2, |f|^2 (Parseval weights)
 
+    const bool cost = CM && mode == ROWS_COST;             // G1 and G2 alone
+    const int qtot = cost ? Cfg::QTOT / 2 : Cfg::QTOT;
     if (issuer) {
         // ---- the chunk stream: product q / NCH (C, E, C, E), K-chunk q % NCH.  One
         // thread: bulk copy of each DFT-matrix chunk two ahead, the products of each
@@ -277,7 +279,7 @@ __global__ void __launch_bounds__(XT_THREADS, 1) k_rows_tc(CurveDev c, int mode,
             int issued_b = 1, waited_b = -1;
             issue_b(0);
             issue_b(1);
-            for (int q = 0; q < Cfg::QTOT; ++q) {
+            for (int q = 0; q < qtot; ++q) {
                 const int g = q / Cfg::NCH, cch = q % Cfg::NCH, sa = q & 1, sb = q % XT_BSTAGES;
                 ok = ok && !*vbad;
                 if (ok && !tc::bar_wait(&a_full[sa], (q >> 1) & 1, wb)) ok = false;
@@ -307,7 +309,7 @@ __global__ void __launch_bounds__(XT_THREADS, 1) k_rows_tc(CurveDev c, int mode,
                 }
                 tc::commit(&mma_done[sb]);   // also when nothing was issued: keeps the phases in step
                 // matrix chunk q + 2 into the stage of chunk q - 1, once its products are done
-                if (ok && q + 2 < Cfg::QTOT) {
+                if (ok && q + 2 < qtot) {
                     if (q >= 1 && !tc::bar_wait(&mma_done[(q - 1) % XT_BSTAGES], ((q - 1) / XT_BSTAGES) & 1, wb)) {
                         ok = false;
                         *vbad = 1;
@@ -320,7 +322,7 @@ __global__ void __launch_bounds__(XT_THREADS, 1) k_rows_tc(CurveDev c, int mode,
             }
             // copies that may still be landing (after a wait gave up), and the last products
             for (int qq = waited_b + 1; qq <= issued_b; ++qq) tc::bar_wait(&full_b[qq % XT_BSTAGES], (qq / XT_BSTAGES) & 1);
-            tc::bar_wait(&mma_done[(Cfg::QTOT - 1) % XT_BSTAGES], ((Cfg::QTOT - 1) / XT_BSTAGES) & 1);
+            tc::bar_wait(&mma_done[(qtot - 1) % XT_BSTAGES], ((qtot - 1) / XT_BSTAGES) & 1);
         }
         __syncwarp();
     } else {
@@ -439,7 +441,7 @@ __global__ void __launch_bounds__(XT_THREADS, 1) k_rows_tc(CurveDev c, int mode,
                     s[3] += cw * (ur * ur + ui * ui);
                     s[4] += cw * (fr * fr + fi * fi);
                 }
-                if (has) st_half<CM>(Rrow + cch * XT_KC * cs, cs, rv);
+                if (has && !cost) st_half<CM>(Rrow + cch * XT_KC * cs, cs, rv);
             };
             unsigned u0[XT_HV], d0[XT_HV], w0[XT_HV], u1[XT_HV], d1[XT_HV], w1[XT_HV];
             fu(0, u0);
@@ -465,6 +467,7 @@ __global__ void __launch_bounds__(XT_THREADS, 1) k_rows_tc(CurveDev c, int mode,
 #pragma unroll
             for (int k = 0; k < 5; ++k) hsum[r][k] = s[k];
         }
+        if (!cost) {
         // ---- G3: r_x = (i k r^) C   (r^ as just written by this thread)
         product(fetch_row(Rrow), no_wait, [&](int cch, const unsigned (&rb)[XT_HV], float (&v)[XT_HV]) {
             const int j0 = mode0(cch);
@@ -541,6 +544,7 @@ __global__ void __launch_bounds__(XT_THREADS, 1) k_rows_tc(CurveDev c, int mode,
                 }
                 step(cch + 1, r1, p1);
             }
+        }
         }
         tc::fence_before();
     }
@@ -673,7 +677,8 @@ static cudaError_t rows_tc_dispatch(const CurveDev &c, int mode, cudaStream_t st
 
 cudaError_t launch_rows_tc(const CurveDev &c, int mode, cudaStream_t st, StepArm arm)
 {
-    return c.cc ? rows_tc_dispatch<true>(c, mode, st, arm) : rows_tc_dispatch<false>(c, mode, st, arm);
+    return c.cc ? rows_tc_dispatch<true>(c, mode, st, arm)
+                : rows_tc_dispatch<false>(c, mode == ROWS_COST ? ROWS_EVAL : mode, st, arm);
 }
 
 }  // namespace ks
