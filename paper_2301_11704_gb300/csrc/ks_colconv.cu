@@ -137,10 +137,17 @@ struct TermSum {
     __device__ __forceinline__ double value() const { return sizeof(T) == 8 ? (double)hi : (double)hi + (double)lo; }
 };
 
-// T_k and H_k of one frequency
+// The product's factors at one frequency: with s = +1, Y = (a x + b y, c x + d y) for
+// Z = (x, y), a = T.x + H.x, b = H.y - T.y, c = T.y + H.y, d = T.x - H.x; s = -1 swaps a
+// with d and b with -c.
 template <typename T>
 struct alignas(16) SpecPair {
-    cpx<T> t, h;
+    cpx<T> t, h;   // (a, b), (c, d)
+    __device__ __forceinline__ cpx<T> times(cpx<T> z, bool even) const
+    {
+        if (even) return {t.x * z.x + t.y * z.y, h.x * z.x + h.y * z.y};
+        return {h.y * z.x - h.x * z.y, t.x * z.y - t.y * z.x};
+    }
 };
 __device__ __forceinline__ SpecPair<float> ldc_spec(const SpecPair<float> *p)
 {
@@ -304,7 +311,7 @@ __device__ __forceinline__ void cc_body(const CurveDev &c, int mode, int discret
         // element r carries the quarter twist e^(-2 pi i r / 4E)
         auto put = [&](int r, T z) { v[r] = {z * cos128<T>(U128 * r), -(z * sin128<T>(U128 * r))}; };
         auto get = [&](int r) { return v[r].x * cos128<T>(U128 * r) - v[r].y * sin128<T>(U128 * r); };
-        auto contract = [&](T sg, bool first) {
+        auto contract = [&](bool even, bool first) {
             F::template dif<false, HOIST>(v, buf, tw, tid, sync);
             asm volatile("" ::: "memory");   // the spectra are not loaded ahead of the transform
             // the step's decision, for the epilogue (published by the barriers of dit())
@@ -313,9 +320,7 @@ __device__ __forceinline__ void cc_body(const CurveDev &c, int mode, int discret
 #pragma unroll
             for (int e = 0; e < E; ++e) {
                 const SpecPair<T> p = HOIST ? ldc_spec(spec + e * NT + tid) : spec[e * NT + tid];
-                const cpx<T> t = p.t, h = p.h, z = v[e];
-                const T hx = sg * h.x, hy = sg * h.y;
-                v[e] = {(t.x + hx) * z.x + (hy - t.y) * z.y, (t.y + hy) * z.x + (t.x - hx) * z.y};
+                v[e] = p.times(v[e], even);
             }
             if (DEFER && first && tid == 0) {
                 // CTA 0 decides, which starts first and waits for nobody; bounded all the same
@@ -344,11 +349,11 @@ __device__ __forceinline__ void cc_body(const CurveDev &c, int mode, int discret
         // one or two contractions (a descent step: the update, then D_t u of the updated
         // column) through the same code: unrolled into two copies it outgrew the
         // instruction caches (the warps' largest stall at L = 16384)
-        T sg = discrete ? T(-1) : T(1);
+        bool even = !discrete;
         bool store = !DEFER && mode == GM_STORE;
 #pragma unroll 1
         for (;;) {
-            contract(sg, !store);
+            contract(even, !store);
             if (store) {
                 constexpr int CH = E < 8 ? E : 8;   // row scales loaded a group ahead of the stores
                 T rs[CH];
@@ -432,7 +437,7 @@ __device__ __forceinline__ void cc_body(const CurveDev &c, int mode, int discret
                 const T up = lane < 31 ? nx : (q < E * (NT / 32) ? edge[q] : T(0));
                 put(r, tid + NT * r < P ? up - v[r].x : T(0));
             }
-            sg = T(1);
+            even = true;
             store = true;
         }
     }
@@ -562,8 +567,7 @@ __global__ void __launch_bounds__(F::NT) k_cx(const __grid_constant__ CurveDev c
                 else f(std::integral_constant<int, 3>());
             }
         };
-        T sg = discrete ? T(-1) : T(1);
-        bool store = !DEFER && mode == GM_STORE, first = true;
+        bool even = !discrete, store = !DEFER && mode == GM_STORE, first = true;
 #pragma unroll 1
         for (;;) {
             by_rank([&](auto rk) {
@@ -585,9 +589,7 @@ __global__ void __launch_bounds__(F::NT) k_cx(const __grid_constant__ CurveDev c
 #pragma unroll
             for (int e = 0; e < E; ++e) {
                 const SpecPair<T> p = spec[e * NT + tid];
-                const cpx<T> t = p.t, h = p.h, z = v[e];
-                const T hx = sg * h.x, hy = sg * h.y;
-                v[e] = {(t.x + hx) * z.x + (hy - t.y) * z.y, (t.y + hy) * z.x + (t.x - hx) * z.y};
+                v[e] = p.times(v[e], even);
             }
             F::template dit<true>(v, buf, tw, tid, sync);
             if (first) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -660,7 +662,7 @@ __global__ void __launch_bounds__(F::NT) k_cx(const __grid_constant__ CurveDev c
                     const int n = tid + NT * r + Q * p;
                     d[p][r] = n < P ? ub[n + 1] - ub[n] : T(0);
                 }
-            sg = T(1);
+            even = true;
             store = true;
             first = false;
         }
@@ -845,17 +847,25 @@ __global__ void __launch_bounds__(256) k_cc_specB(const __grid_constant__ CurveS
     }
     __syncthreads();
     const int idx = blockIdx.x * blockDim.x + threadIdx.x;
-    if (idx < 2 * L) {
-        const int kind = idx / L, rank = (idx % L) / F::L, e = (idx % F::L) / F::NT, t = idx % F::NT;
+    if (idx < L) {
+        const int rank = idx / F::L, e = (idx % F::L) / F::NT, t = idx % F::NT;
         const int k = CS * F::freq(t, e) + rank, k1 = k % A, k2 = k / A;
-        const double2 *S = (const double2 *)c.ccx + (size_t)kind * L + (size_t)k1 * B;
-        double re = 0.0, im = 0.0;
-        for (int n2 = 0; n2 < B; ++n2) {
-            const double2 w = wB[(n2 * k2) & (B - 1)], x = S[n2];
-            re += x.x * w.x - x.y * w.y;
-            im += x.x * w.y + x.y * w.x;
+        const double2 *S = (const double2 *)c.ccx + (size_t)k1 * B;
+        double2 x[2];
+#pragma unroll
+        for (int kind = 0; kind < 2; ++kind) {
+            double re = 0.0, im = 0.0;
+            for (int n2 = 0; n2 < B; ++n2) {
+                const double2 w = wB[(n2 * k2) & (B - 1)], y = S[(size_t)kind * L + n2];
+                re += y.x * w.x - y.y * w.y;
+                im += y.x * w.y + y.y * w.x;
+            }
+            x[kind] = make_double2(re / L, im / L);
         }
-        ((cpx<T> *)c.ccs)[2 * (rank * F::L + e * F::NT + t) + kind] = {(T)(re / L), (T)(im / L)};
+        SpecPair<T> o;   // T in x[0], H in x[1]
+        o.t = {(T)(x[0].x + x[1].x), (T)(x[1].y - x[0].y)};
+        o.h = {(T)(x[0].y + x[1].y), (T)(x[0].x - x[1].x)};
+        ((SpecPair<T> *)c.ccs)[rank * F::L + e * F::NT + t] = o;
     }
     if (idx < F::TW * CS) {
         long long num, den;
@@ -902,7 +912,7 @@ cudaError_t setup_spectra(const CurveSet &cs, int nc, cudaStream_t st)
     constexpr int L = F::L * CS;
     int A = 1;
     while (A * A < L) A <<= 1;
-    const int B = L / A, n = 2 * L > F::TW * CS ? 2 * L : F::TW * CS;
+    const int B = L / A, n = L > F::TW * CS ? L : F::TW * CS;
     for (int o = 0; o < nc; o += GRID_Y) {
         const CurveSet part = cs.from(o);
         const int k = nc - o < GRID_Y ? nc - o : GRID_Y;

@@ -187,7 +187,7 @@ struct RegFft {
     // or runs of lr(i) elements) fall in distinct banks
     static constexpr int PSH = sizeof(T) == 4 ? 4 : 3;
     static constexpr bool PAD2 = sizeof(T) == 4 && L > 256 && lr(1) == 8 && sub(1) == 256;
-    static __device__ __forceinline__ int ph(int p)
+    static __host__ __device__ constexpr int ph(int p)
     {
         int q = p + (p >> PSH);
         if constexpr (PAD2) q += (p >> 8) * 8;
@@ -235,9 +235,11 @@ struct RegFft {
     {
 #pragma unroll
         for (int b = 0; b < E / rad(I); ++b) {
-            const int p = pos0<I>(tid, b);
+            // p and lr r have no bit in common, so their places in the padded buffer add: one
+            // address per butterfly, the elements at constant offsets
+            const cpx<T> *q = buf + ph(pos0<I>(tid, b));
 #pragma unroll
-            for (int r = 0; r < rad(I); ++r) v[b * rad(I) + r] = buf[ph(p + lr(I) * r)];
+            for (int r = 0; r < rad(I); ++r) v[b * rad(I) + r] = q[ph(lr(I) * r)];
         }
     }
     template <int I>
@@ -245,9 +247,9 @@ struct RegFft {
     {
 #pragma unroll
         for (int b = 0; b < E / rad(I); ++b) {
-            const int p = pos0<I>(tid, b);
+            cpx<T> *q = buf + ph(pos0<I>(tid, b));
 #pragma unroll
-            for (int r = 0; r < rad(I); ++r) buf[ph(p + lr(I) * r)] = v[b * rad(I) + r];
+            for (int r = 0; r < rad(I); ++r) q[ph(lr(I) * r)] = v[b * rad(I) + r];
         }
     }
     template <int I, bool CONJ, bool NC>
