@@ -22,15 +22,25 @@ namespace ks {
 
 namespace {
 
-// V = 1: the plan of FP64 curves with few sections
+// V = 0: the plan of batches and of single curves that fill the chip with it; V = 1, 2:
+// fewer values per thread, for single curves of few sections (cm_warps, cm_spread).
+// N = 128 in FP32 keeps 8 values throughout: 16 were slower at every size (17.0 us a
+// step instead of 20.2 at N_s = 4096, 47.9 instead of 49.7 at 16384, a batch of 256
+// curves 0.555 ms instead of 0.567).
 template <typename T, int N, int V = 0>
 struct RowFft;
 template <> struct RowFft<float, 8> { using F = RegFft<float, 8, 2, false, true, 2, 2, 2>; };
 template <> struct RowFft<float, 16> { using F = RegFft<float, 16, 4, false, true, 4, 4>; };
 template <> struct RowFft<float, 32> { using F = RegFft<float, 32, 8, false, true, 8, 4>; };
 template <> struct RowFft<float, 64> { using F = RegFft<float, 64, 8, false, true, 8, 8>; };
-template <> struct RowFft<float, 128> { using F = RegFft<float, 128, 16, false, true, 16, 8>; };
+template <> struct RowFft<float, 128> { using F = RegFft<float, 128, 8, false, true, 8, 8, 2>; };
 template <> struct RowFft<float, 256> { using F = RegFft<float, 256, 16, false, true, 16, 16>; };
+template <> struct RowFft<float, 32, 1> { using F = RegFft<float, 32, 2, false, true, 2, 2, 2, 2, 2>; };
+template <> struct RowFft<float, 64, 1> { using F = RegFft<float, 64, 2, false, true, 2, 2, 2, 2, 2, 2>; };
+template <> struct RowFft<float, 128, 1> { using F = RegFft<float, 128, 4, false, true, 4, 4, 4, 2>; };
+template <> struct RowFft<float, 256, 1> { using F = RegFft<float, 256, 8, false, true, 8, 8, 4>; };
+template <> struct RowFft<float, 32, 2> { using F = RegFft<float, 32, 4, false, true, 4, 4, 2>; };
+template <> struct RowFft<float, 64, 2> { using F = RegFft<float, 64, 4, false, true, 4, 4, 4>; };
 // FP64: 4 values per thread (8 at N = 256): a warp's FP64 instruction holds its pipe for
 // about 64 cycles whatever the size of the curve, so the work is spread over warps
 template <> struct RowFft<double, 32> { using F = RegFft<double, 32, 4, false, true, 4, 4, 2>; };
@@ -394,11 +404,11 @@ __device__ __forceinline__ void rows_cm_body(const CurveDev &c, int mode, int bl
     rows_finish<NTHR>(c, mode, nblk, true, arm);
 }
 
-// Four CTAs of N = 256 FP32 sections per SM (128 registers a thread): 2.2 waves of
-// three become 1.7 of four at N_s = 16384.
+// FP32: 16 warps per SM at 16 values a thread (128 registers): N = 256 and N_s = 16384
+// in 1.7 waves instead of 2.2.  20 at fewer (96 registers, no spills to speak of).
 template <typename T, int N, int SEC, int V>
 __global__ void __launch_bounds__(CmCfg<T, T, N, SEC, V>::NTHR,
-                                  sizeof(T) == 4 && N >= 128 ? 512 / CmCfg<T, T, N, SEC, V>::NTHR : 1)
+                                  sizeof(T) == 4 && N >= 128 ? (N == 128 || V ? 640 : 512) / CmCfg<T, T, N, SEC, V>::NTHR : 1)
     k_rows_cm(const __grid_constant__ CurveDev c, int mode, StepArm arm)
 {
     if ((int)blockIdx.x == c.row_blocks) {   // the extra CTA of the deferred form
@@ -618,6 +628,22 @@ cudaError_t cm_dispatch(int n, int sec, Fn &&f)
     });
 }
 
+// Warps of a single curve's row phase on a plan.  FP32 curves run on the plan of the
+// fewest values per thread that has at most CM_WARPS of them, 8 per SM: below that the
+// phase is one wave bound by the chain of a warp and by the first pass through its code,
+// both of which shrink with the values per thread; above, by the instructions in all,
+// which grow.  Graph step in us on the finer / the coarser plan: N = 64, 2 and 4 values,
+// 9.4 / 9.9 at N_s = 1024, 11.7 / 11.9 at 2048, 15.5 / 14.8 at 3000; 4 and 8 values,
+// 15.2 / 15.4 at 4096, 26.0 / 25.9 at 6000; N = 128, 4 and 8 values, 10.6 / 12.2 at 1024,
+// 17.2 / 16.6 at 3000; N = 256, 8 and 16 values, 14.4 / 18.0 at 1024, 17.1 / 20.0 at 2048,
+// 24.9 / 25.0 at 4096, 96.6 / 94.9 at 16384.
+constexpr int CM_WARPS = 1216;
+template <typename T, int N, int V>
+constexpr int cm_warps(int ns)
+{
+    return (ns + 1) / 2 * RowFft<T, N, V>::F::NT / 32;
+}
+
 template <typename T, int N, int SEC, int V>
 cudaError_t rows_run(const CurveDev &c, int mode, cudaStream_t st, StepArm arm)
 {
@@ -634,6 +660,10 @@ cudaError_t rows_t(const CurveDev &c, int mode, cudaStream_t st, StepArm arm)
     }
     return cm_dispatch<T>(c.nx, c.rsec, [&](auto nn, auto ss) {
         constexpr int N = decltype(nn)::value, SEC = decltype(ss)::value;
+        if constexpr (sizeof(T) == 4 && N >= 32)
+            if (cm_warps<T, N, 1>(c.ns) <= CM_WARPS) return rows_run<T, N, SEC, 1>(c, mode, st, arm);
+        if constexpr (sizeof(T) == 4 && (N == 32 || N == 64))
+            if (cm_warps<T, N, 2>(c.ns) <= CM_WARPS) return rows_run<T, N, SEC, 2>(c, mode, st, arm);
         return rows_run<T, N, SEC, 0>(c, mode, st, arm);
     });
 }

@@ -72,6 +72,13 @@ def test_column_form_matches_dense(precision, N, Ns):
     _compare(_curves(N, Ns, precision), precision)
 
 
+# the sections at which single FP32 curves change the row phase's values per thread
+@pytest.mark.parametrize("N,Ns", [(32, 4866), (32, 4867), (32, 9735), (64, 2432), (64, 2433), (64, 4866), (64, 4867),
+                                  (128, 2432), (128, 2433), (256, 2432), (256, 2433)])
+def test_row_plans_match_dense(N, Ns):
+    _compare(_curves(N, Ns, "fp32"), "fp32", steps=2)
+
+
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
 @pytest.mark.parametrize("symmetry", [0, 1, 3, 5, 7])
 @pytest.mark.parametrize("adjoint", ["paper", "discrete"])
