@@ -67,6 +67,16 @@ __device__ __forceinline__ void it_put8(unsigned char *stage, int part_bytes, in
     *reinterpret_cast<uint4 *>(stage + part_bytes + it_kmaj(row, k0)) = make_uint4(w1[0], w1[1], w1[2], w1[3]);
 }
 
+// The same for two values of the row, k0 a multiple of 2.
+__device__ __forceinline__ void it_put2(unsigned char *stage, int part_bytes, int row, int k0, const float (&x)[2])
+{
+    const __nv_bfloat162 h = __floats2bfloat162_rn(x[0], x[1]);
+    const float2 hf = __bfloat1622float2(h);
+    const __nv_bfloat162 l = __floats2bfloat162_rn(x[0] - hf.x, x[1] - hf.y);
+    *reinterpret_cast<__nv_bfloat162 *>(stage + it_kmaj(row, k0)) = h;
+    *reinterpret_cast<__nv_bfloat162 *>(stage + part_bytes + it_kmaj(row, k0)) = l;
+}
+
 // Row tiles and K chunks of a parity block of n rows (padded with zeros).
 __host__ __device__ inline int it_tiles(int n) { return (n + IT_M - 1) / IT_M; }
 __host__ __device__ inline int it_chunks(int n) { return (n + IT_KC - 1) / IT_KC; }
@@ -178,7 +188,36 @@ __global__ void __launch_bounds__(IT_THREADS, 1) k_imp_tc(CurveDev c, int splits
     // splits and writes the operand stage.
     constexpr int UNITS = N * (IT_KC / 8), UPT = (UNITS + IT_THREADS - 1) / IT_THREADS;
     const float *Bsrc = FWD ? G : Y;
+    // Column-major sources: a warp's item is 8 columns by 8 sections, two sections per
+    // thread (lane % 4) of column lane / 4, so that a load touches 8 runs of a sector
+    // instead of 32 and the 4-byte stores fall in distinct banks (the row-major units below
+    // took the increment of a step at N_s = 4096, N = 128 to 127 us on such sources, 73 on
+    // row-major ones; N = 128, N_s = 4096 now steps in 106 us, 121 with row-major fields).
+    const bool cm = rs == 1;
+    const int lane = tid & 31;
+    auto cm_item = [&](int q, int i, int &col, int &k) {   // false: past the last item
+        const int v = warp + (IT_THREADS / 32) * i;
+        col = 8 * (v >> 2) + (lane >> 2);
+        k = q * IT_KC + 8 * (v & 3) + 2 * (lane & 3);
+        return v < N / 2;
+    };
     auto fetch = [&](int q, float (&xa)[UPT][8], float (&xb)[UPT][8]) {
+        if (cm) {
+#pragma unroll
+            for (int j = 0; j < UPT; ++j)
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    int col, k;
+                    bool v = cm_item(q, 4 * j + e / 2, col, k);
+                    k += e & 1;
+                    v = v && k < np;
+                    const int ra = FWD ? 1 + k : k;
+                    const int rb = (p == 0 && k >= h) ? ra : M - k;
+                    xa[j][e] = v ? Bsrc[ra + col * cs] : 0.f;
+                    xb[j][e] = (FWD && v) ? G[rb + col * cs] : 0.f;
+                }
+            return;
+        }
 #pragma unroll
         for (int j = 0; j < UPT; ++j) {
             const int u = tid + j * IT_THREADS, col = u % N, kb = u / N, k0 = q * IT_KC + 8 * kb;
@@ -194,6 +233,23 @@ __global__ void __launch_bounds__(IT_THREADS, 1) k_imp_tc(CurveDev c, int splits
         }
     };
     auto produce = [&](int q, unsigned char *bst, const float (&xa)[UPT][8], const float (&xb)[UPT][8]) {
+        if (cm) {
+#pragma unroll
+            for (int j = 0; j < UPT; ++j)
+#pragma unroll
+                for (int e = 0; e < 8; e += 2) {
+                    int col, k;
+                    if (!cm_item(q, 4 * j + e / 2, col, k)) continue;
+                    float x[2];
+#pragma unroll
+                    for (int i = 0; i < 2; ++i) {
+                        const float a = xa[j][e + i], b = xb[j][e + i];
+                        x[i] = !FWD ? a : p ? r2 * (a - b) : k + i < h ? r2 * (a + b) : a;
+                    }
+                    it_put2(bst, Cfg::B_PART, col, k & (IT_KC - 1), x);
+                }
+            return;
+        }
 #pragma unroll
         for (int j = 0; j < UPT; ++j) {
             const int u = tid + j * IT_THREADS, col = u % N, kb = u / N, k0 = q * IT_KC + 8 * kb;

@@ -79,6 +79,13 @@ def test_row_plans_match_dense(N, Ns):
     _compare(_curves(N, Ns, "fp32"), "fp32", steps=2)
 
 
+# the implicit increment's tensor-core products on column-major operands, K ranges that end
+# inside a chunk (M odd and even), every N they are built for
+@pytest.mark.parametrize("N,Ns", [(32, 68), (64, 301), (128, 131), (256, 194)])
+def test_implicit_on_columns_matches_dense(N, Ns):
+    _compare(_curves(N, Ns, "fp32", scheme="implicit"), "fp32", steps=3)
+
+
 @pytest.mark.parametrize("precision", ["fp64", "fp32"])
 @pytest.mark.parametrize("symmetry", [0, 1, 3, 5, 7])
 @pytest.mark.parametrize("adjoint", ["paper", "discrete"])
