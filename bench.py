@@ -475,9 +475,8 @@ def implicit_context(dev, timed_steps, K, dtau=0.5):
 
 def symmetric_context(dev, timed_steps, K):
     """Curves held in the odd subspace (Sec. V.B: real parts of every section's
-    coefficients zero) beside the general run: symmetry = 1 keeps full storage
-    (the three-launch four-step form then transforms the imaginary columns of two
-    modes as one sequence); symmetry = 5 keeps only the sine coefficients (half
+    coefficients zero) beside the general run: symmetry = 1 keeps full storage;
+    symmetry = 5 keeps only the sine coefficients (half
     the field bytes, half the columns of every s-contraction).  The L=44,
     N_x=128, N_s=4096 FP32 curve and the L=22, N_x=64, N_s=1024 curve in FP32 and
     FP64."""
@@ -589,7 +588,9 @@ def run_curve(args):
     fx, fs, fpw = flops_per_point(N, M)
     F = curve.fft_length
     form = curve.s_form
-    fused = form == "fft4c" and "dt_store" not in prof
+    # one launch for both contractions: the column form (k_cc: reads r^, A^ and U, writes U
+    # and D) or the cluster form of an explicit s_transform
+    one_launch = "dt_update" in prof and "dt_store" not in prof
     kernels = {}   # name -> (mean ms per launch, algorithmic bytes, algorithmic flops, traffic kind)
     rows_kind = "rows_tc" if precision.startswith("bf16") else "rows"
     if "rows" in prof:
@@ -601,13 +602,15 @@ def run_curve(args):
     chained = form == "fft4"
     for key, nb in (("dt_update", 4.0), ("dt_store", 1.0 if chained else 2.0)):
         if key in prof:
-            fl = fs / 2 * M * (2 if (key == "dt_update" and fused) else 1)
-            by = (nb + (2.0 if (key == "dt_update" and fused) else 0.0)) * N * b * spec.Ns
+            both = key == "dt_update" and one_launch
+            fl = fs / 2 * M * (2 if both else 1)
+            by = (nb + (1.0 if both else 0.0)) * N * b * spec.Ns
             kernels[key] = (prof[key]["ms"] / prof[key]["launches"], by, fl, "fft4")
     dom = max(kernels, key=lambda k: kernels[k][0])
     t_dom, by_dom, fl_dom, kind = kernels[dom]
     kernel_names = {"rows": "row phase (k_rows%s)" % ("_tc" if rows_kind == "rows_tc" else ""),
-                    "dt_update": "update contraction (%s)" % form, "dt_store": "D_t u contraction (%s)" % form}
+                    "dt_update": ("both contractions and the update (%s)" % ("k_cc" if args.s_transform == "auto" else form)
+                                  if one_launch else "update contraction (%s)" % form), "dt_store": "D_t u contraction (%s)" % form}
     ach = by_dom / (t_dom / 1e3) / 1e9
     roof = {"bound": "hbm", "achieved": ach, "peak": hbm_peak, "unit": "GB/s", "frac": ach / hbm_peak,
             "traffic": None, "peak_source": peak_src + " (MEASURED_PEAKS.json hbm_gbs)",
@@ -627,7 +630,7 @@ def run_curve(args):
     traf = None
     if dom == "rows":
         traf = recorded_traffic("rows:%s:N%d:Ns%d:%s" % (rows_kind, N, spec.Ns, precision), rows_kind)
-    elif form == "fft4":
+    elif form == "fft4" and not one_launch:
         traf = recorded_traffic("%s:fft4:N%d:Ns%d:%s" % (dom, N, spec.Ns, precision), "fft4")
     if traf:
         roof["traffic"] = traf["bytes_per_launch"]
@@ -662,7 +665,7 @@ def run_curve(args):
         nbytes = spec.Ns * N * b
         # every step: the curve from pinned host memory (set_state), one descent
         # step, and its result J read back to the host (ks_curve_descend copies the
-        # device scalar record, 176 bytes, and synchronises).  Two device buffers:
+        # device scalar record, 192 bytes, and synchronises).  Two device buffers:
         # the next step's copy runs on a copy stream while this step computes (the
         # buffer it fills was last read by the step before, which has completed).
         cur = torch.cuda.current_stream(dev)
@@ -686,7 +689,7 @@ def run_curve(args):
         torch.cuda.synchronize(dev)
         e2e_s = time.perf_counter() - t0
         e2e = {"value": M * n_e2e / e2e_s, "unit": UNIT, "h2d_bytes_per_step": nbytes,
-               "d2h_bytes_per_step": 176, "steps": n_e2e,
+               "d2h_bytes_per_step": 192, "steps": n_e2e,
                "path": "pinned host curve -> set_state -> descend(1), J read back; each step's host-to-device "
                        "copy overlaps the step before (two device buffers, a copy stream)"}
     sc = curve.scalars()
@@ -757,7 +760,9 @@ def run_curve(args):
                "seconds_per_step_estimates": est}
 
     if rank == 0:
-        launches = {"fft4": 7, "fft4c": 2 if fused else 3}.get(form, 3)
+        # the row phase, the contractions (one launch each or one for both) and, in the column
+        # form, the closing sum of |G|^2 of each call
+        launches = (3 if args.s_transform == "auto" else 2) if one_launch else {"fft4": 7}.get(form, 3)
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": K, "warmup": W,
                 "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
                 "vs_baseline": None, "dtype": {"fp64": "f64", "fp32": "f32"}.get(precision, precision + "+f32"),
