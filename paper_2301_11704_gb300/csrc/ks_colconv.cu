@@ -474,6 +474,11 @@ __device__ __forceinline__ void cc_body(const CurveDev &c, int mode, int discret
     }
 }
 
+// Bound: at few sections the chain of a column's stages and their barriers (N_x = 64,
+// N_s = 1024 FP32, both contractions of a step and its reduction: 10.8 us, where the
+// clustered four-step kernel took 21.3); at many, issue slots (N_x = 256, N_s = 16384:
+// 70 us, half of the issue slots used, FMA pipe 35%, 50 MB read from DRAM where the
+// three-launch form took 132 + 69 us); in FP64 the FP64 pipes (83% busy in a batch).
 // Up to 128 registers a thread: at 32 values per thread the transform's 64 registers
 // of data, its twiddles and the epilogue about fit.
 template <class F, bool DEFER>
@@ -493,7 +498,8 @@ __global__ void __launch_bounds__(F::NT, F::NT >= 512 ? 1 : 512 / F::NT)
 // and owns the sections [rank Q, (rank + 1) Q): the classes' parts of q at n + p Q go to
 // CTA p through distributed shared memory, the updated sections to every CTA.  For
 // FP64 curves of few columns, whose CTAs would leave most SMs idle while each is
-// bound by its FP64 pipes.
+// bound by its FP64 pipes: N_x = 64, N_s = 552 over two CTAs a step in 45 us, over one
+// in 64 (143 before the column form); the pipes of the SMs in use are then 77% busy.
 template <class F, int CS>
 constexpr size_t cx_bytes() { return F::BYTES + ((size_t)(CS - 1) * F::L + CS * F::L + 1) * sizeof(typename F::type); }
 
@@ -697,7 +703,10 @@ __global__ void __launch_bounds__(F::NT) k_cx(const __grid_constant__ CurveDev c
     }
 }
 
-// Batched curves: work item (curve, column) per CTA, the curves of one length.
+// Batched curves: work item (curve, column) per CTA, the curves of one length.  A step
+// of the 256-curve batch (N_x 32 to 128, N_s 256 to 2048), contractions and row phase:
+// FP32 0.555 ms (1.49 with the four-step form), bound by issue slots and shared memory;
+// FP64 11.6 ms (17.1), by the FP64 pipes.
 template <class F>
 __global__ void __launch_bounds__(F::NT, F::NT >= 512 ? 1 : 512 / F::NT) k_cc_batch(const CurveDev *cv, const int2 *items,
                                                                                     int mode, int discrete, int gate)

@@ -34,7 +34,6 @@ __device__ __forceinline__ cpx<T> cmul(cpx<T> a, cpx<T> b)
 // no CTA leaves before it.  No kernel triggers its successor early: successor
 // CTAs parked on the SMs during a whole kernel slowed graph replay (measured).
 // A no-op for a kernel launched without the attribute.
-__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Arrival of a CTA at a grid-wide last-CTA reduction, after the CTA has written

@@ -1,6 +1,10 @@
 // ks_kernels.cu -- sm_103a kernels of one adjoint-descent step for a curve of
 // KSE states (Ashtari & Schneider, arXiv 2301.11704).
 //
+// Curves of the column form (`auto` from N_s = 64 to 16384 in FP32 and 8192 in FP64) run
+// on column-major fields in two kernels per step, ks_rows_cm.cu (or ks_rows_tc.cu) and
+// ks_colconv.cu; what follows is the row-major path of the other forms.
+//
 // Data layout (every field): row-major [N_s][N] real words of the storage type T.
 // Row m holds section s_m spectrally: N/2 complex Fourier coefficients
 // u^_{m,j}, j = 0..N/2-1, interleaved (re, im); the Nyquist coefficient is not

@@ -11,8 +11,13 @@
 // column accesses and row accesses both fall in distinct banks.  Two real sections
 // are packed into one complex transform of N points, held by N / E threads in
 // registers (ks_rfft.cuh): the physical section u stays in registers between the
-// products, and a transform crosses shared memory once (N <= 128 and N = 256 in
-// FP32) or twice.
+// products, and a transform crosses shared memory once to three times.
+//
+// Bound: at few sections the chain of a warp (N = 64, N_s = 1024 FP32 8.5 us alone, the
+// row-major warp transforms 12.8; N = 128, N_s = 4096 10.8 and 18.0); at many, the
+// shared-memory pipe and the round trips to memory between its phases (N = 256,
+// N_s = 16384 36 us and 66, 67 MB of fields at 1.9 TB/s); in FP64 the FP64 pipes (N = 64,
+// N_s = 4096 42 us and 64).
 #include <type_traits>
 
 #include "ks_dfloat.cuh"
@@ -605,7 +610,8 @@ cudaError_t cm_launch(void (*kern)(KArgs...), int grid, int block, size_t smem, 
 }
 
 // FP64 single curves on the plan of 2 values per thread: about a warp or less for each
-// of the SMs' 608 quarters (a warp holds one pair at N = 64, two at N = 32)
+// of the SMs' 608 quarters (a warp holds one pair at N = 64, two at N = 32).  An FP64
+// instruction holds a quarter's pipe, so a second warp there would wait for the first.
 bool cm_spread(int nx, int ns) { return (nx == 64 && ns <= 1216) || (nx == 32 && ns <= 2432); }
 
 // The section counts built: 4 (FP64), 8 and 16, where a CTA has at least one warp.
