@@ -91,8 +91,10 @@ Layout make_layout(int ns, int nx, int prec, int allow_split, int bn, int s_tran
     l.pitch = cc_pitch(ns);
     l.single = allow_split;
     l.ccl = l.cc && allow_split ? cc_cluster(l.cc, w, prec) : 1;
-    // sections per row-phase CTA: fewer where the curve has few sections (the FP64 work,
-    // and latency, want every SM), 64-byte runs of a column where it has many
+    // sections per row-phase CTA: 64-byte runs of a column where the curve has many (FP32,
+    // 16 against 8, step in us: N_s = 4096 at N = 256 24.9 / 26.3, 16384 97.4 / 102.9; FP64,
+    // 8 against 4: within 2% either way from N_s = 2500 to 8192), fewer below N_s = 2048,
+    // where they leave SMs idle
     l.rsec = l.cc ? cm_sections(nx, ns, prec, prec ? (ns >= 2048 ? 16 : 8) : (ns >= 2048 ? 8 : 4), allow_split) : 0;
     size_t field = l.cc ? al256((size_t)w * l.pitch * b) : al256((size_t)ns * w * b);
     // tiling and split of the s-contraction (over the w stored columns)
