@@ -80,12 +80,11 @@ class KSBatch:
         return [o.as_dict() for o in out]
 
     def get_state(self, i: int) -> torch.Tensor:
+        """Physical state of curve i, complete when this returns (on any stream)."""
         s = self.specs[i]
         out = torch.empty((s.Ns, s.N), dtype=self.dtype, device=self.device)
         check(self.lib.ks_batch_get_state(self.handle, int(i), out.data_ptr()))
-        # on torch's current stream the tensor's readers are ordered after the copy
-        if self.stream != torch.cuda.current_stream(self.device):
-            self.stream.synchronize()
+        self.stream.synchronize()
         return out
 
     def autotune(self, steps: int = 8) -> dict:
