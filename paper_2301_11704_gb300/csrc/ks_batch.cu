@@ -667,9 +667,9 @@ ks_status ks_batch_autotune(ks_batch *b, int32_t steps, int32_t *chosen)
         }
         if (s == KS_OK) s = set_split(kv.first, best_f1);
     }
-    // knob 3: the column tile of dense-form curves with N >= 64
+    // knob 3: the column tile of dense-form curves with N >= 64 (neither FFT nor column form)
     bool dense = false;
-    for (int i = 0; i < b->nb; ++i) dense = dense || (b->cv[i].F == 0 && b->cv[i].W >= 64);
+    for (int i = 0; i < b->nb; ++i) dense = dense || (!b->cv[i].cc && b->cv[i].F == 0 && b->cv[i].W >= 64);
     if (dense && s == KS_OK) {
         int best_t = b->tile_pref;
         for (int t : {64, 32}) {

@@ -29,3 +29,22 @@ def test_get_state_returns_a_finished_copy():
     b.get_state(0)
     assert b.stream.query()
     b.close()
+
+
+def test_autotune_leaves_the_dense_tile_without_dense_curves():
+    """Column-form curves have no s-phase tile: the row phase's two widths (2 + 3 steps
+    each) are all that is timed, on the callers' curves."""
+    b, _ = _batch(_four_step_specs([(64, 300), (128, 400)]), precision="fp32")
+    tune = b.autotune(3)
+    assert tune["dense_tile"] == 0
+    assert [x["step"] for x in b.scalars()] == [10, 10]
+    b.close()
+
+
+def test_autotune_tries_the_dense_tile_of_dense_curves():
+    """One dense curve (N_s = 40) of 64 columns beside a column-form one: both widths are timed."""
+    b, _ = _batch(_four_step_specs([(64, 40), (64, 300)]), precision="fp32", s_transform="dense")
+    tune = b.autotune(3)
+    assert tune["dense_tile"] in (32, 64)
+    assert [x["step"] for x in b.scalars()] == [20, 20]
+    b.close()
