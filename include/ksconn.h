@@ -382,7 +382,7 @@ ks_status ks_batch_get_state(ks_batch *b, int32_t i, void *u_dev);
 ks_status ks_batch_autotune(ks_batch *b, int32_t steps, int32_t *chosen);
 
 typedef struct {
-    int32_t row_sections;   /* sections per row-phase CTA */
+    int32_t row_sections;   /* sections per row-phase CTA (of the column-form curves where there are some) */
     int32_t dense_tile;     /* s-phase tile width of dense-form curves (0: per-curve default) */
     int32_t nlen;           /* transform lengths of the four-step curves (at most 8 listed) */
     int32_t F[8], F1[8];    /* each length F and its split F = F1 (F / F1) */

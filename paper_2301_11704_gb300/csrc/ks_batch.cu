@@ -49,7 +49,8 @@ struct ks_batch {
     Group imp_prod{}, imp_fin{};        // its items: the two products, the finishing pass
     std::map<int, int> named;           // column-form curves: the transform length and split their sizes name
     int tile_pref = 0;                  // 0: per-curve default, 32 or 64: forced (autotuner)
-    int row_warps = ks::ROWS_WARPS;     // warps per row-phase CTA (two sections each): 4 or 8 (autotuner)
+    int row_warps = ks::ROWS_WARPS;     // row-major curves: warps per row-phase CTA (two sections each), 4 or 8 (autotuner)
+    int col_sections = ks::ROWS_PER_CTA; // column-form curves: sections per row-phase CTA, 8 or 16 (autotuner)
     float tuned_ms = 0.f;               // the autotuner's time of a step with its choice
     cudaGraphExec_t gexec = nullptr;
     cudaStream_t gstream = nullptr;
@@ -127,7 +128,7 @@ ks_status build_items(ks_batch *b)
     std::map<std::pair<int, int>, std::vector<int2>> fft;   // by (F, F1): each group launched with its own shared memory
     for (int i = 0; i < b->nb; ++i) {
         ks::CurveDev &c = b->cv[i];
-        if (c.cc) c.rsec = ks::cm_sections(c.nx, c.ns, b->prec, 2 * b->row_warps, 0);
+        if (c.cc) c.rsec = ks::cm_sections(c.nx, c.ns, b->prec, b->col_sections, 0);
         const int rs = c.cc ? c.rsec : 2 * b->row_warps;
         c.row_blocks = (c.ns + rs - 1) / rs;
         for (int k = 0; k < c.row_blocks; ++k) rows[c.nx + (c.cc ? CM_KEY : 0)].push_back(make_int2(i, k));
@@ -214,11 +215,14 @@ static cudaError_t launch_fft_group(const ks_batch *b, const Group &g, int mode,
     return ks::launch_sconv_batch(b->prec, g.key, b->cv_dev, items, g.count, mode, discrete, 1, st);
 }
 
+// as reported: of the column-form curves where there are some
+static int row_sections(const ks_batch *b) { return b->ccs.empty() ? 2 * b->row_warps : b->col_sections; }
+
 static cudaError_t launch_rows_group(const ks_batch *b, const Group &g, int mode, cudaStream_t st)
 {
     const int2 *items = (const int2 *)(b->items_dev + g.off);
     if (g.key >= CM_KEY)
-        return ks::launch_rows_cm_batch(b->prec, g.key - CM_KEY, 2 * b->row_warps, b->cv_dev, items, g.count, mode, st);
+        return ks::launch_rows_cm_batch(b->prec, g.key - CM_KEY, b->col_sections, b->cv_dev, items, g.count, mode, st);
     return ks::launch_rows_batch(b->prec, g.key, b->row_warps, b->cv_dev, items, g.count,
                                  mode == ks::ROWS_COST ? ks::ROWS_EVAL : mode, st);
 }
@@ -354,7 +358,7 @@ ks_status init_all(ks_batch *b, int npert, const double *amps_host, const double
     }
     for (const Group &g : b->rows)
         if (e == cudaSuccess && g.key >= CM_KEY)
-            e = ks::launch_trial_batch_cm(b->prec, g.key - CM_KEY, 2 * b->row_warps, b->cv_dev,
+            e = ks::launch_trial_batch_cm(b->prec, g.key - CM_KEY, b->col_sections, b->cv_dev,
                                           (const int2 *)(b->items_dev + g.off), g.count, npert, amps, vp, vo, b->st);
     for (const Group &g : b->ccs)
         if (e == cudaSuccess)
@@ -475,8 +479,8 @@ ks_status ks_batch_create(int32_t nb, const ks_params *params, const double *u_p
     b->nb = nb;
     b->prec = ks::storage32(params[0].precision);
     b->discrete = params[0].adjoint == KS_ADJ_DISCRETE;
-    // FP32: 16 sections per row CTA (64-byte runs of a column; 6% of the 256-curve step)
-    if (b->prec) b->row_warps = 2 * ks::ROWS_WARPS;
+    // FP32 columns: 16 sections per row CTA (64-byte runs of a column; 6% of the 256-curve step)
+    if (b->prec) b->col_sections = 2 * ks::ROWS_PER_CTA;
     b->impl = params[0].scheme == KS_SCHEME_IMPLICIT;
     b->st = (cudaStream_t)stream;
     cudaGetDevice(&b->device);
@@ -644,13 +648,15 @@ ks_status ks_batch_autotune(ks_batch *b, int32_t steps, int32_t *chosen)
     ks_status s = KS_OK;
     float best = 1e30f, ms = 0.f;
     // knob 1: sections per row-phase CTA
-    int best_w = b->row_warps;
+    int best_w = b->row_warps, best_c = b->col_sections;
     for (int w : {ks::ROWS_WARPS, 2 * ks::ROWS_WARPS}) {
         b->row_warps = w;
+        b->col_sections = 2 * w;
         if ((s = time_steps(&ms)) != KS_OK) break;
-        if (ms < best) { best = ms; best_w = w; }
+        if (ms < best) { best = ms; best_w = w; best_c = 2 * w; }
     }
     b->row_warps = best_w;
+    b->col_sections = best_c;
     // knob 2: the split of each length of the four-step curves
     std::map<int, int> lens;   // F -> current F1
     for (int i = 0; i < b->nb && s == KS_OK; ++i)
@@ -684,7 +690,7 @@ ks_status ks_batch_autotune(ks_batch *b, int32_t steps, int32_t *chosen)
     if (s != KS_OK) return s;
     b->tuned_ms = best / (float)steps;
     s = build_items(b);
-    if (chosen) *chosen = 2 * b->row_warps;
+    if (chosen) *chosen = row_sections(b);
     return s;
 }
 
@@ -692,7 +698,7 @@ ks_status ks_batch_get_tuning(ks_batch *b, ks_batch_tuning *out)
 {
     if (!b || !out) return ks::report_error(KS_EINVAL, "batch handle and out are required");
     *out = ks_batch_tuning{};
-    out->row_sections = 2 * b->row_warps;
+    out->row_sections = row_sections(b);
     out->dense_tile = b->tile_pref;
     std::map<int, int> lens = b->named;
     for (int i = 0; i < b->nb; ++i)

@@ -48,3 +48,12 @@ def test_autotune_tries_the_dense_tile_of_dense_curves():
     assert tune["dense_tile"] in (32, 64)
     assert [x["step"] for x in b.scalars()] == [20, 20]
     b.close()
+
+
+@pytest.mark.parametrize("form,precision,sections", [("auto", "fp32", 16), ("auto", "fp64", 8), ("dense", "fp32", 8),
+                                                     ("fft", "fp32", 8), ("dense", "fp64", 8)])
+def test_row_sections_of_a_new_batch(form, precision, sections):
+    """16 sections per row CTA only where FP32 curves run the column form."""
+    b, _ = _batch(_four_step_specs([(64, 300), (128, 400)]), precision=precision, s_transform=form)
+    assert b.tuning()["row_sections"] == sections
+    b.close()
