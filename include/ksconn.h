@@ -425,9 +425,12 @@ ks_status ks_cost_noalloc(const ks_params *p, const void *u_dev, double *out_dev
 
 /* Test hook for the failure path of the device-side bounded waits; the paper has
  * no counterpart.  The kernels that wait on an mbarrier (the split-BF16 row
- * phase, the FFT form with one CTA per mode, the tensor-core contraction) spin
+ * phase, the FFT form with one CTA per mode, the tensor-core contraction) or, in
+ * the column form of a single curve, for the step's convergence decision spin
  * at most `cycles` clock cycles in their first wait of a launch (0 restores the
- * default, about 2^31 cycles; a negative value makes that wait give up at once).
+ * default, about 2^31 cycles; a negative value makes that wait give up at once:
+ * the decision is then withheld from the columns that wait for it, and the step
+ * is not applied).
  * A wait that gives up sets the curve's error word, lets the copies and
  * products already in flight finish (with the default bound), frees its tensor
  * memory and returns; every later call that reads the curve's scalars returns

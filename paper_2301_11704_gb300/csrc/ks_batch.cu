@@ -323,7 +323,7 @@ ks_status read_all(ks_batch *b, std::vector<ks::DevScalars> &h)
     if (e != cudaSuccess) return ks::report_error(KS_ECUDA, "scalar read: %s", cudaGetErrorString(e));
     for (size_t i = 0; i < h.size(); ++i)
         if (h[i].err)
-            return ks::report_error(KS_ETIMEOUT, "curve %zu: a device-side copy did not complete in time", i);
+            return ks::report_error(KS_ETIMEOUT, "curve %zu: a device-side wait ran out", i);
     return KS_OK;
 }
 

@@ -148,7 +148,7 @@ ks_status read_scalars(ks_curve *c, ks::DevScalars *h)
 {
     KS_CUDA(cudaMemcpyAsync(h, c->d.sc, sizeof(*h), cudaMemcpyDeviceToHost, c->st));
     KS_CUDA(cudaStreamSynchronize(c->st));
-    if (h->err) return fail(KS_ETIMEOUT, "a device-side copy did not complete in time; re-initialise the curve");
+    if (h->err) return fail(KS_ETIMEOUT, "a device-side wait ran out; re-initialise the curve");
     return KS_OK;
 }
 

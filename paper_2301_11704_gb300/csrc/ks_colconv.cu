@@ -179,6 +179,7 @@ __device__ __forceinline__ void cc_decide(const CurveDev &c, int tid)
     double a0 = 0.0, a1 = 0.0, a2 = 0.0;
     const double tol = sc->tol;
     const int conv = sc->conv;
+    const bool withheld = sc->wait_cycles < 0;   // test hook: every column's wait runs out
     if (w < FW) {
 #pragma unroll 4
         for (int b = w * 32 + lane; b < c.row_parts; b += FW * 32) {
@@ -204,7 +205,8 @@ __device__ __forceinline__ void cc_decide(const CurveDev &c, int tid)
         for (int k = 0; k < FW; ++k) r += red[k][lane];
     const double j2 = __shfl_sync(0xffffffffu, r, 0), num = __shfl_sync(0xffffffffu, r, 1), den = __shfl_sync(0xffffffffu, r, 2);
     auto publish = [&](bool stop) {
-        if (lane == 0) asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(&sc->decided), "r"(stop ? 2 : 1) : "memory");
+        if (lane == 0 && !withheld)
+            asm volatile("st.relaxed.gpu.global.s32 [%0], %1;" ::"l"(&sc->decided), "r"(stop ? 2 : 1) : "memory");
     };
     // without a tolerance: finite, with no quotient (den = 0 gives J_arc = 0) unless it may overflow
     const bool quick = tol <= 0 && isfinite(j2) && (fabs(num) < 1e300 * den);
@@ -251,6 +253,20 @@ __device__ __forceinline__ int cc_decided(const DevScalars *sc)
     int d;
     asm volatile("ld.relaxed.gpu.global.s32 %0, [%1];" : "=r"(d) : "l"(&sc->decided) : "memory");
     return d;
+}
+
+// The wait for it where a first look (d) found none: CTA 0 decides, which starts first and
+// waits for nobody; bounded all the same.  A step that is not decided in time is not
+// applied and flagged as error 6; where only some columns gave up they differ by a step
+// from the others, and the curve has to be initialised again.
+__device__ __forceinline__ bool cc_wait(DevScalars *sc, int d)
+{
+    if (d == 0) {
+        const long long t0 = clock64(), lim = wait_bound(*sc);
+        while ((d = cc_decided(sc)) == 0 && clock64() - t0 < lim) {}
+        if (d == 0) atomicExch(&sc->err, 6);
+    }
+    return d == 1;
 }
 
 // DEFER: a single curve's fused step (mode GM_STEP) after a row phase that left its
@@ -322,15 +338,7 @@ __device__ __forceinline__ void cc_body(const CurveDev &c, int mode, int discret
                 const SpecPair<T> p = HOIST ? ldc_spec(spec + e * NT + tid) : spec[e * NT + tid];
                 v[e] = p.times(v[e], even);
             }
-            if (DEFER && first && tid == 0) {
-                // CTA 0 decides, which starts first and waits for nobody; bounded all the same
-                if (d == 0) {
-                    const long long t0 = clock64(), lim = wait_bound(*sc);
-                    while ((d = cc_decided(sc)) == 0 && clock64() - t0 < lim) {}
-                    if (d == 0) atomicExch(&sc->err, 6);
-                }
-                go = d == 1;
-            }
+            if (DEFER && first && tid == 0) go = cc_wait(sc, d);
             F::template dit<true, HOIST>(v, buf, tw, tid, sync);
         };
 #pragma unroll
@@ -600,12 +608,9 @@ __global__ void __launch_bounds__(F::NT) k_cx(const __grid_constant__ CurveDev c
             F::template dit<true>(v, buf, tw, tid, sync);
             if (first) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
             if (DEFER && first && rank == 0 && tid == 0) {
-                // CTA 0 decides, which starts first and waits for nobody; bounded all the same.
-                // One answer for the cluster: no CTA leaves while another writes to it.
-                const long long t0 = clock64(), lim = wait_bound(*sc);
-                while (dec == 0 && (dec = cc_decided(sc)) == 0 && clock64() - t0 < lim) {}
-                if (dec == 0) atomicExch(&sc->err, 6);
-                for (int p = 0; p < CS; ++p) *cluster.map_shared_rank(&go, p) = dec == 1;
+                // one answer for the cluster: no CTA leaves while another writes to it
+                const int answer = cc_wait(sc, dec);
+                for (int p = 0; p < CS; ++p) *cluster.map_shared_rank(&go, p) = answer;
             }
             // this class's part of q at its own sections, and at the others' to their CTAs
             T y[E];
