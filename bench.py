@@ -100,6 +100,11 @@ def spec_of(workload):
     return gen.workload(WORKLOADS[workload])[0]
 
 
+def form_of(curve):
+    """The form of the s-contraction that the curve runs."""
+    return "column" if curve.column_length else curve.s_form
+
+
 def workload_name(spec, precision):
     prec = {"fp64": "FP64", "fp32": "FP32 storage and transforms, FP64 reductions",
             "bf16x2": "FP32 storage, x-transforms as 2-term split-BF16 tensor-core products, FP64 reductions",
@@ -493,7 +498,7 @@ def symmetric_context(dev, timed_steps, K):
                         device=dev)
             c.init_trial(0.0, None, amps, vp)
             ms, prof = timed_steps(c, K, 3, profile=K)
-            r[name] = {"ms_per_step": sum(ms) / K, "s_form": c.s_form, "workspace_bytes": c.workspace_bytes,
+            r[name] = {"ms_per_step": sum(ms) / K, "s_form": form_of(c), "workspace_bytes": c.workspace_bytes,
                        "phases_ms": {k: v["ms"] / v["launches"] for k, v in prof.items()
                                      if isinstance(v, dict) and v.get("launches")}}
             c.close()
@@ -586,8 +591,8 @@ def run_curve(args):
     peak_alu = peak_fp32 if b == 4 else 1.25
     hbm_peak = float(peaks["hbm_gbs"])
     fx, fs, fpw = flops_per_point(N, M)
-    F = curve.fft_length
-    form = curve.s_form
+    F = curve.column_length or curve.fft_length
+    form = form_of(curve)
     # one launch for both contractions: the column form (k_cc: reads r^, A^ and U, writes U
     # and D) or the cluster form of an explicit s_transform
     one_launch = "dt_update" in prof and "dt_store" not in prof
@@ -608,8 +613,8 @@ def run_curve(args):
             kernels[key] = (prof[key]["ms"] / prof[key]["launches"], by, fl, "fft4")
     dom = max(kernels, key=lambda k: kernels[k][0])
     t_dom, by_dom, fl_dom, kind = kernels[dom]
-    kernel_names = {"rows": "row phase (k_rows%s)" % ("_tc" if rows_kind == "rows_tc" else ""),
-                    "dt_update": ("both contractions and the update (%s)" % ("k_cc" if args.s_transform == "auto" else form)
+    kernel_names = {"rows": "row phase (k_rows%s)" % ("_tc" if rows_kind == "rows_tc" else "_cm" if form == "column" else ""),
+                    "dt_update": ("both contractions and the update (%s)" % ("k_cc" if form == "column" else form)
                                   if one_launch else "update contraction (%s)" % form), "dt_store": "D_t u contraction (%s)" % form}
     ach = by_dom / (t_dom / 1e3) / 1e9
     roof = {"bound": "hbm", "achieved": ach, "peak": hbm_peak, "unit": "GB/s", "frac": ach / hbm_peak,
@@ -703,7 +708,7 @@ def run_curve(args):
             k64 = max(3, min(20, K))
             ms64, _ = timed_steps(c64, k64, 3)
             ctx["fp64_gpu_path"] = {"value": M * k64 / (sum(ms64) / 1e3), "unit": UNIT,
-                                    "ms_per_step": sum(ms64) / k64, "steps": k64, "s_form": c64.s_form}
+                                    "ms_per_step": sum(ms64) / k64, "steps": k64, "s_form": form_of(c64)}
             c64.close()
         # ---- the other precisions of this workload
         others = {}
@@ -740,7 +745,7 @@ def run_curve(args):
             msd, _ = timed_steps(cd, kd, 3)
             ctx["diff_workload_fp32"] = {"workload": "L=%g N_x=%d N_s=%d FP32" % (sd.L, sd.N, sd.Ns),
                                          "value": sd.M * kd / (sum(msd) / 1e3), "unit": UNIT,
-                                         "ms_per_step": sum(msd) / kd, "steps": kd, "s_form": cd.s_form}
+                                         "ms_per_step": sum(msd) / kd, "steps": kd, "s_form": form_of(cd)}
             cd.close()
         # ---- full-linear-implicit stepping (Sec. V.C.3) on the single large curve
         try:
@@ -762,7 +767,7 @@ def run_curve(args):
     if rank == 0:
         # the row phase, the contractions (one launch each or one for both) and, in the column
         # form, the closing sum of |G|^2 of each call
-        launches = (3 if args.s_transform == "auto" else 2) if one_launch else {"fft4": 7}.get(form, 3)
+        launches = (3 if form == "column" else 2) if one_launch else {"fft4": 7}.get(form, 3)
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": K, "warmup": W,
                 "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
                 "vs_baseline": None, "dtype": {"fp64": "f64", "fp32": "f32"}.get(precision, precision + "+f32"),

@@ -202,17 +202,22 @@ int32_t ks_version(void);
  * matrix is stored: D_t is generated from an O(N_s) table on the fly. */
 size_t ks_curve_workspace_bytes(const ks_params *p);
 
-/* Length of the FFT that a single curve with parameters p applies D_t with
- * (s_transform rule above), or 0 when it uses the dense contraction.  -1 when
- * p is invalid (message in ks_last_error). */
+/* Length of the FFT of the form that a single curve's parameters p name
+ * (ks_curve_s_form), or 0 when that is a dense contraction.  -1 when p is
+ * invalid (message in ks_last_error). */
 int32_t ks_curve_fft_length(const ks_params *p);
 
 /* The form a size names under the rule above, as an s_transform code with `auto`
- * resolved among the codes below (where `auto` runs the column form, the code and
- * ks_curve_fft_length still name the size's other form): 1 dense, 2 FFT with one CTA per mode, 3 dense on the
- * tensor cores, 4 four-step FFT in three launches, 5 four-step FFT in one
- * clustered launch.  -1 when p is invalid (message in ks_last_error). */
+ * resolved among the codes below: 1 dense, 2 FFT with one CTA per mode, 3 dense on
+ * the tensor cores, 4 four-step FFT in three launches, 5 four-step FFT in one
+ * clustered launch.  -1 when p is invalid (message in ks_last_error).  It is the form
+ * that runs, and ks_curve_fft_length its length, where ks_curve_column_length is 0. */
 int32_t ks_curve_s_form(const ks_params *p);
+
+/* Length of the column form's transform where that is what a curve with parameters p
+ * runs (`auto`, from N_s = 64 up to 16384 in FP32 storage and 8192 in FP64), else 0:
+ * the form of ks_curve_s_form runs.  -1 when p is invalid. */
+int32_t ks_curve_column_length(const ks_params *p);
 
 /* Creates a curve (Sec. V.C.1-2).
  *  p            parameters (copied).

@@ -337,6 +337,12 @@ int32_t ks_curve_s_form(const ks_params *p)
     return l.tc ? 3 : 1;
 }
 
+int32_t ks_curve_column_length(const ks_params *p)
+{
+    if (validate(p) != KS_OK) return -1;
+    return ks::curve_layout(p, p->launch == 1).cc;
+}
+
 ks_status ks_curve_create(const ks_params *p, const double *u_plus_host, const double *u_minus_host,
                           const void *u_init_dev, void *workspace_dev, size_t workspace_bytes, void *stream,
                           ks_curve **out)

@@ -45,13 +45,16 @@ class KSCurve:
     bytes and half the columns of every s-contraction; FP64 or FP32, nx >= 16,
     s_transform "auto", "dense", "fft", "fft4" or "fft4c").
     s_transform: how D_t is applied along s (same results to rounding): "auto"
-    (the form measured fastest for the size), "dense", "dense_tc" (FP32, tensor
+    (the form measured fastest for the size: the column form from ns = 64 to 16384 in
+    FP32 and 8192 in FP64), "dense", "dense_tc" (FP32, tensor
     cores), "fft" (one CTA per mode; four-step above its limit), "fft4" (four-step
-    FFT, three launches), "fft4c" (four-step FFT, one clustered launch); the form
-    in use is in `s_form`, the FFT length in `fft_length`.
+    FFT, three launches), "fft4c" (four-step FFT, one clustered launch).  The
+    column form's transform length is in `column_length`, 0 where another form runs:
+    then the form in use is in `s_form` and its FFT length in `fft_length` (which
+    name one of these forms for every size).
     launch: "auto" / "kernels" run descent steps as kernels per phase (row phase
-    and the two contractions; one launch for both contractions in the clustered
-    form), "persistent" runs many steps of a dense-form curve in one cooperative
+    and the two contractions; one launch for both contractions in the column and the
+    clustered form), "persistent" runs many steps of a dense-form curve in one cooperative
     kernel (same results; slower on GB300 at the sizes measured).
     scheme: "imex" takes only the diagonal term -a_j^2 u of G implicitly (stable
     while dtau rho(lambda^2 D_t^2) < 2); "implicit" every linear term of G,
@@ -77,7 +80,9 @@ class KSCurve:
         if nbytes == 0:
             raise _native.KSError(_native.KS_EINVAL, self.lib.ks_last_error().decode())
         self.workspace_bytes = int(nbytes)
-        # length of the FFT that applies D_t along s (0: dense contraction)
+        # the column form's length (0: the form of s_form runs), and the form the size names
+        # with the length of its FFT (0: dense contraction)
+        self.column_length = int(self.lib.ks_curve_column_length(ctypes.byref(self.params)))
         self.fft_length = int(self.lib.ks_curve_fft_length(ctypes.byref(self.params)))
         self.s_form = _FORM_NAME.get(int(self.lib.ks_curve_s_form(ctypes.byref(self.params))))
         # descent steps run as one persistent kernel (dense form) or as three kernels per step

@@ -53,7 +53,7 @@ def main(argv=None):
     sc = c.scalars()
     c.close()
     out = {"L": sp.L, "N_x": sp.N, "N_s": sp.Ns, "precision": args.precision,
-           "fft_length": c.fft_length, "ms_per_step": ms, "J": sc["J"]}
+           "column_length": c.column_length, "fft_length": c.fft_length, "ms_per_step": ms, "J": sc["J"]}
     if phases is not None:
         out["ms_per_phase_launch"] = phases
     print(json.dumps(out))
