@@ -317,9 +317,10 @@ __device__ __forceinline__ bool cc_wait(DevScalars *sc, int d)
     return d == 1;
 }
 
-// DEFER: a single curve's fused step (mode GM_STEP) after a row phase that left its
-// reduction here; else the modes of launch_dt with their own last-CTA reduction.
-template <class F, bool DEFER>
+// DEFER: a single curve's step (mode GM_STEP) after a row phase that left its reduction
+// here; else GM_GRAD, GM_STORE and in a batch (BATCH) GM_STEP, with their own last-CTA
+// reduction.
+template <class F, bool DEFER, bool BATCH = false>
 __device__ __forceinline__ void cc_body(const CurveDev &c, int mode, int discrete, int gate, int col, int ncol)
 {
     using T = typename F::type;
@@ -349,7 +350,7 @@ __device__ __forceinline__ void cc_body(const CurveDev &c, int mode, int discret
     T *D = as_global((T *)c.D + co), *U = as_global((T *)c.U + co), *G = as_global((T *)c.G + co);
     const T *A = as_global((const T *)c.A + co), *R = as_global((const T *)c.R + co);
     const T *wt = (const T *)c.wt, *rowscale = (const T *)c.ccr;
-    const bool step = DEFER || mode == GM_STEP, upd = step || mode == GM_UPDATE;
+    const bool step = DEFER || (BATCH && mode == GM_STEP);
     double partsum = 0.0;
 
     // the first contraction's column: section n + 1 beside n
@@ -399,7 +400,7 @@ __device__ __forceinline__ void cc_body(const CurveDev &c, int mode, int discret
             for (int r = 0; r < E; ++r) {
                 const int n = tid + NT * r;
                 a[EARLY ? r : 0] = n < ns ? A[n] : T(0);
-                u[EARLY ? r : 0] = (upd && n < ns) ? U[n] : T(0);
+                u[EARLY ? r : 0] = (step && n < ns) ? U[n] : T(0);
             }
         }
         // one or two contractions (a descent step: the update, then D_t u of the updated
@@ -446,7 +447,7 @@ __device__ __forceinline__ void cc_body(const CurveDev &c, int mode, int discret
                     rs[i] = ok ? tab(rowscale + n) : T(0);
                     w[i] = ok ? tab(wt + n) : T(0);
                     av[i] = EARLY ? a[EARLY ? r0 + i : 0] : (ok ? A[n] : T(0));
-                    uv[i] = EARLY ? u[EARLY ? r0 + i : 0] : ((upd && ok) ? U[n] : T(0));
+                    uv[i] = EARLY ? u[EARLY ? r0 + i : 0] : ((step && ok) ? U[n] : T(0));
                 }
             };
             fetch(0);
@@ -469,7 +470,7 @@ __device__ __forceinline__ void cc_body(const CurveDev &c, int mode, int discret
                     const T g = interior ? -(ac[i] + lam * y) : T(0);
                     if constexpr (sizeof(T) == 8) sum.add(wc[i], g);
                     else gc[i] = g;
-                    if (upd) {
+                    if (step) {
                         const T un = uc[i] + dtp * g;   // the end rows unchanged (g = 0)
                         if (interior) U[n] = un;
                         v[r].x = un;
@@ -522,7 +523,7 @@ __device__ __forceinline__ void cc_body(const CurveDev &c, int mode, int discret
         t = warp_sum(t);
         if (lane == 0) {
             sc->G2 = c.L * t;
-            if (upd) {
+            if (step) {
                 sc->step += 1;
                 sc->tau += sc->dtau;
                 sc->lambda = sc->lambda_next;
@@ -558,6 +559,7 @@ __global__ void __launch_bounds__(F::NT, F::NT >= 512 ? 1 : 512 / F::NT)
 // FP64 curves of few columns, whose CTAs would leave most SMs idle while each is
 // bound by its FP64 pipes: N_x = 64, N_s = 552 over two CTAs a step in 45 us, over one
 // in 64 (143 before the column form); the pipes of the SMs in use are then 77% busy.
+// DEFER: a step (mode GM_STEP); else GM_GRAD or GM_STORE.
 template <class F, int CS>
 constexpr size_t cx_bytes() { return F::BYTES + ((size_t)(CS - 1) * F::L + CS * F::L + 1) * sizeof(typename F::type); }
 
@@ -591,12 +593,11 @@ __global__ void __launch_bounds__(F::NT) k_cx(const __grid_constant__ CurveDev c
     const T *wt = as_global((const T *)c.wt), *rowscale = as_global((const T *)c.ccr);
     const cpx<T> *tw = as_global((const cpx<T> *)c.cctw + (size_t)rank * F::TW);
     const SpecPair<T> *spec = as_global((const SpecPair<T> *)c.ccs + (size_t)rank * Q);
-    const bool step = DEFER || mode == GM_STEP, upd = step || mode == GM_UPDATE;
     double partsum = 0.0;
 
     if (!col_live(col, c.sym, c.hs)) {   // held at zero (the whole cluster)
         if (DEFER && rank == 0 && col == 1 - c.hs) cc_decide<NT>(c, tid);
-        if (mode == GM_STORE || step)
+        if (DEFER || mode == GM_STORE)
             for (int j = rank * NT + tid; j < ns; j += CS * NT) D[j] = T(0);
         if (mode == GM_GRAD)
             for (int j = rank * NT + tid; j < ns; j += CS * NT) G[j] = T(0);
@@ -619,7 +620,7 @@ __global__ void __launch_bounds__(F::NT) k_cx(const __grid_constant__ CurveDev c
             for (int r = 0; r < E; ++r) {
                 const int n = n0 + NT * r;
                 a[r] = n < ns ? A[n] : T(0);
-                u[r] = (upd && n < ns) ? U[n] : T(0);
+                u[r] = (DEFER && n < ns) ? U[n] : T(0);
             }
         }
         cpx<T> v[E];
@@ -700,7 +701,7 @@ __global__ void __launch_bounds__(F::NT) k_cx(const __grid_constant__ CurveDev c
                 const bool interior = n > 0 && n < P;
                 const T g = interior ? -(a[r] + lam * y[r]) : T(0);
                 sum.add(n < ns ? wt[n] : T(0), g);
-                if (upd) {
+                if (DEFER) {
                     u[r] += dtp * g;   // the end rows unchanged (g = 0)
                     if (interior) U[n] = u[r];
                 } else if (n < ns) {
@@ -708,7 +709,7 @@ __global__ void __launch_bounds__(F::NT) k_cx(const __grid_constant__ CurveDev c
                 }
             }
             partsum = (col_mode(col, c.hs) == 0 ? 1.0 : 2.0) * sum.value();
-            if (!step) break;
+            if constexpr (!DEFER) break;
 #pragma unroll
             for (int p = 0; p < CS; ++p) {
                 T *dst = cluster.map_shared_rank(ub, p);
@@ -748,11 +749,6 @@ __global__ void __launch_bounds__(F::NT) k_cx(const __grid_constant__ CurveDev c
         t = warp_sum(t);
         if (lane == 0) {
             sc->G2 = c.L * t;
-            if (upd) {
-                sc->step += 1;
-                sc->tau += sc->dtau;
-                sc->lambda = sc->lambda_next;
-            }
             sc->cnt_gemm = 0;
         }
     }
@@ -768,7 +764,7 @@ __global__ void __launch_bounds__(F::NT, F::NT >= 512 ? 1 : 512 / F::NT) k_cc_ba
 {
     const int2 it = items[blockIdx.x];
     const CurveDev &c = cv[it.x];
-    cc_body<F, false>(c, mode, discrete, gate, it.y, c.W);
+    cc_body<F, false, true>(c, mode, discrete, gate, it.y, c.W);
 }
 
 __global__ void k_cc_finish(const __grid_constant__ CurveDev c)
@@ -1097,6 +1093,8 @@ cudaError_t launch_setup_cc_spectra(int prec, int L, const CurveDev *cv, const i
 
 cudaError_t launch_cc(const CurveDev &c, int mode, int discrete, int gate, cudaStream_t st)
 {
+    // a single curve's step is deferred (the implicit scheme has GM_GRAD in its place)
+    if (mode != GM_GRAD && mode != GM_STORE && !(mode == GM_STEP && c.defer)) return cudaErrorInvalidValue;
     if (c.ccl > 1) return run_cx(c, mode, discrete, gate, st);
     return c.prec ? run_t<float>(c, mode, discrete, gate, st) : run_t<double>(c, mode, discrete, gate, st);
 }

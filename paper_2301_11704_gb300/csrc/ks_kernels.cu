@@ -1305,7 +1305,6 @@ cudaError_t launch_row_fwd_x(const CurveDev &c, void *spec, int keep_ends, cudaS
 
 cudaError_t launch_row_fwd(const CurveDev &c, const void *phys, void *spec, cudaStream_t st)
 {
-    if (c.cc) return launch_row_fwd_cm(c, phys, spec, SetScalars{0.0, 0.0, 0}, st);
     return c.prec ? row_fwd_t<float, dfloat, float>(c, phys, spec, 0, st)
                   : row_fwd_t<double, double, double>(c, phys, spec, 0, st);
 }
