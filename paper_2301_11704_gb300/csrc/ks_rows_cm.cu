@@ -432,15 +432,19 @@ __global__ void __launch_bounds__(CmCfg<T, T, N, SEC>::NTHR) k_rows_cm_batch(con
     rows_cm_body<T, N, SEC>(c, mode, it.y, c.row_blocks, StepArm{0, 0.0, 0});
 }
 
-// e^(-2 pi i k / N), k < N / 2, in the transform's type
+// e^(-2 pi i k / N), k < N / 2, in the transform's type (FP32: the nearest values, not
+// the row phase's pairs of modulus 1: a state read back has the smaller error with them)
 template <typename T>
 __device__ __forceinline__ cpx<T> row_root(const CurveDev &c, int k)
 {
     if constexpr (std::is_same<T, dfloat>::value) {
         const float4 w = ((const float4 *)c.twdf)[k];
         return {dfloat(w.x, w.y), dfloat(w.z, w.w)};
+    } else if constexpr (sizeof(T) == 4) {
+        const float4 w = ((const float4 *)c.twdf)[k];
+        return {w.x, w.z};
     } else {
-        return ((const cpx<T> *)(sizeof(T) == 8 ? c.twid64 : c.twid))[k];
+        return ((const cpx<T> *)c.twid64)[k];
     }
 }
 
