@@ -47,10 +47,11 @@ namespace {
 
 // The transform of each length (B: of batched curves).  FP32: 16 values per thread, 32
 // from L = 8192 on (two exchanges instead of three: 35.7 against 43.6 us a step's
-// contraction at 256 x 8000), 8 up to L = 512 and for single curves up to 2048, which
-// are bound by the latency of a column's chain (L = 1024: 10.7 against 12.9 us; the
+// contraction at 256 x 8000), 8 at L = 256 and 512 and for single curves up to 2048,
+// which are bound by the latency of a column's chain (L = 1024: 10.7 against 12.9 us; the
 // 256-curve batch, bound by throughput, takes 0.74 ms a step with 8 and 0.57 with
-// 16).  FP64: few values, to give every quarter of an SM's FP64 pipes a warp.
+// 16), and 4 at L = 128, a warp.  FP64: few values, to give every quarter of an SM's FP64
+// pipes a warp: 2 to 8, 16 at L = 8192.
 template <typename T, int L, bool B = false>
 struct CcPlan : CcPlan<T, L, false> {};
 template <> struct CcPlan<float, 128, false> { using F = RegFft<float, 128, 4, true, false, 4, 4, 4, 2>; };
@@ -73,7 +74,8 @@ template <> struct CcPlan<double, 8192, false> { using F = RegFft<double, 8192, 
 
 // The split form (a column over a cluster of CS CTAs): the transform of one class of
 // L / CS frequencies.  A warp's FP64 instruction takes about 64 cycles on its quarter
-// of the SM, so the plans give every quarter a warp: 4 values per thread (2 at 256).
+// of the SM, so the plans give every quarter a warp: 2 values per thread at 256, 4 at 512
+// and 1024, 8 at 2048 and 4096.
 template <int Q>
 struct CxPlan;
 template <> struct CxPlan<256> { using F = RegFft<double, 256, 2, true, true, 2, 2, 2, 2, 2, 2, 2, 2>; };

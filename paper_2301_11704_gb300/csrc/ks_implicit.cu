@@ -340,9 +340,11 @@ ks_status setup_implicit(const CurveDev &c, cudaStream_t st)
 //                 U's update, and the step's bookkeeping in the last CTA.
 // The products are register-tiled on the CUDA cores, K in steps of 16 through shared
 // memory.  FP32: 128 x 64 outputs per CTA, 8 x 4 per thread.  FP64: 32 x 32 per CTA,
-// 4 x 2 per thread: the FP64 pipes (2 FMAs a cycle and SM) bound the product whatever
-// the tile, so it is cut fine enough to reach every SM (128 x 64 tiles put the paper's
-// M = 550, N = 64 on 24 of 152: 190 us a product, 32 x 32 on 144).
+// 4 x 2 per thread, cut fine enough to reach every SM: 128 x 64 tiles put the paper's
+// M = 550, N = 64 on 24 of 152 (190 us a product), 32 x 32 on 144 (40 us).  The FMAs alone
+// would take 16 us there (2 a cycle and SM); padded tiles and K chunks of unlike length
+// make 20 of them; the rest has not been taken apart (a barrier on either side of each
+// stage with one CTA per SM, the implicit factor's division in every split's epilogue).
 constexpr int IM_THREADS = 256;   // of the elementwise passes
 template <typename T>
 struct ImCfg {

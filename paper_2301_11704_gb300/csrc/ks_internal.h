@@ -128,7 +128,9 @@ inline int cc_size(int ns, int prec)
 // 256 to 4096 frequencies.  W columns over 1 / 2 / 4 CTAs, step in us: W = 32, N_s = 1024
 // 63 / 44 / 34, 4096 234 / 133 / 84; W = 64, N_s = 552 64 / 45 / 46, 4096 250 / 149 / 158;
 // W = 128, N_s = 552 74 / 76 / 85, 1500 136 / 140 / 150: as many CTAs as reach every SM
-// (W CTAs <= 152, so W <= 38 and 76), and no more.
+// (W CTAs <= 152, so W <= 38 and 76), and no more.  FP32 curves take one CTA per column:
+// the split form is built in FP64 only, where a column is bound by its SM's pipes; an
+// FP32 column is a chain of stages, and what a split would make of it is not measured.
 inline int cc_cluster(int L, int w, int prec)
 {
     if (prec) return 1;

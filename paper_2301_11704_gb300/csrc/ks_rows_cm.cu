@@ -29,9 +29,9 @@ namespace {
 
 // V = 0: the plan of batches and of single curves that fill the chip with it; V = 1, 2:
 // fewer values per thread, for single curves of few sections (cm_warps, cm_spread).
-// N = 128 in FP32 keeps 8 values throughout: 16 were slower at every size (17.0 us a
-// step instead of 20.2 at N_s = 4096, 47.9 instead of 49.7 at 16384, a batch of 256
-// curves 0.555 ms instead of 0.567).
+// V = 0 at N = 128 in FP32: 8 values, 16 were slower at every size (a step with 8 and
+// with 16: 17.0 and 20.2 us at N_s = 4096, 47.9 and 49.7 at 16384, a batch of 256 curves
+// 0.555 and 0.567 ms).
 template <typename T, int N, int V = 0>
 struct RowFft;
 template <> struct RowFft<float, 8> { using F = RegFft<float, 8, 2, false, true, 2, 2, 2>; };
@@ -46,7 +46,7 @@ template <> struct RowFft<float, 128, 1> { using F = RegFft<float, 128, 4, false
 template <> struct RowFft<float, 256, 1> { using F = RegFft<float, 256, 8, false, true, 8, 8, 4>; };
 template <> struct RowFft<float, 32, 2> { using F = RegFft<float, 32, 4, false, true, 4, 4, 2>; };
 template <> struct RowFft<float, 64, 2> { using F = RegFft<float, 64, 4, false, true, 4, 4, 4>; };
-// FP64: 4 values per thread (8 at N = 256): a warp's FP64 instruction holds its pipe for
+// FP64, N = 32 to 128: 4 values per thread: a warp's FP64 instruction holds its pipe for
 // about 64 cycles whatever the size of the curve, so the work is spread over warps
 template <> struct RowFft<double, 32> { using F = RegFft<double, 32, 4, false, true, 4, 4, 2>; };
 template <> struct RowFft<double, 64> { using F = RegFft<double, 64, 4, false, true, 4, 4, 4>; };
@@ -55,7 +55,8 @@ template <> struct RowFft<double, 128> { using F = RegFft<double, 128, 4, false,
 // pair's chain, a fifth more instructions in all)
 template <> struct RowFft<double, 32, 1> { using F = RegFft<double, 32, 2, false, true, 2, 2, 2, 2, 2>; };
 template <> struct RowFft<double, 64, 1> { using F = RegFft<double, 64, 2, false, true, 2, 2, 2, 2, 2, 2>; };
-// double-float (and the FP64 lengths not listed): 8 values per thread
+// double-float, and the FP64 lengths not listed above: 2, 4 and from N = 32 on 8 values
+// per thread
 template <typename T> struct RowFft<T, 8> { using F = RegFft<T, 8, 2, false, true, 2, 2, 2>; };
 template <typename T> struct RowFft<T, 16> { using F = RegFft<T, 16, 4, false, true, 4, 4>; };
 template <typename T> struct RowFft<T, 32> { using F = RegFft<T, 32, 8, false, true, 8, 4>; };
