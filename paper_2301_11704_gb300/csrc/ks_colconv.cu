@@ -120,72 +120,37 @@ auto cc_dispatch(int L, Fn &&fn, decltype(fn(typename CcPlan<T, 128, B>::F())) n
     return none;
 }
 
-// Sum of a thread's terms w g^2: FP64 in FP64 storage; in FP32 storage a compensated
-// FP32 pair (Knuth's TwoSum), which keeps the sum of the FP32 terms to about 2^-46
-// without the FP64 pipe (its issue rate is a small fraction of the FP32 one).  The
-// terms keep the range of g: w reaches S P / pi, so w g^2 leaves FP32's long before
-// g^2 does.  A thread with few values (ALL: they come in one call) scales them by the
-// power of two that brings their largest to [1, 4) and the sum back in FP64; with 32, in
-// groups, one with a term outside [2^-100, 2^100] goes to the FP64 pipe (no curve at
-// its usual scale has one).  The branch took 5 to 9% of a step of the short plans,
-// whose chain waits for instructions at each jump; the scaling takes 0.3 to 1.3%.
-template <typename T, bool ALL>
-struct TermSum {   // T = double
-    T sum = T(0);
-    __device__ __forceinline__ void add(T w, T g) { sum += w * (g * g); }
-    __device__ __forceinline__ double value() const { return sum; }
-};
-template <bool ALL>
-struct TermSum<float, ALL> {
+// Sum of a thread's E terms w(r) g(r)^2 in FP32 storage: a compensated FP32 pair (Knuth's
+// TwoSum), which keeps the sum of the FP32 terms to about 2^-46 without the FP64 pipe (its
+// issue rate is a small fraction of the FP32 one).  The terms keep the range of g: w
+// reaches S P / pi, so w g^2 leaves FP32's long before g^2 does.  They are scaled by the
+// power of two that brings the largest g^2 to [1, 4), and the sum is scaled back in FP64.
+// (Terms out of range to FP64 behind a branch took 5 to 9% of a step of the short plans,
+// whose chain waits for instructions at each jump; the scaling 0 to 1.3%.)
+template <int E, typename W, typename G>
+__device__ __forceinline__ double sum_terms(W &&w, G &&g)
+{
+    float m[E];
+#pragma unroll
+    for (int r = 0; r < E; ++r) m[r] = fabsf(g(r));
+#pragma unroll
+    for (int o = E / 2; o > 0; o >>= 1)
+#pragma unroll
+        for (int r = 0; r < o; ++r) m[r] = fmaxf(m[r], m[r + o]);
+    // the scale's exponent field: 2^(127 - e) for the field e of the largest
+    const int f = max(254 - (int)(__float_as_uint(m[0]) >> 23), 1);
+    const float scale = __uint_as_float((unsigned)f << 23);
     float hi = 0.f, lo = 0.f;
-    double far = 0.0, unit = 1.0;
-    __device__ __forceinline__ void pair(float t)
-    {
-        const float s = __fadd_rn(hi, t), b = __fsub_rn(s, hi);
+#pragma unroll
+    for (int r = 0; r < E; ++r) {
+        const float q = g(r) * scale, t = w(r) * (q * q), s = __fadd_rn(hi, t), b = __fsub_rn(s, hi);
         lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(t, b)));
         hi = s;
     }
-    template <int C>
-    __device__ __forceinline__ void add(const float (&w)[C], const float (&g)[C])
-    {
-        if constexpr (ALL) {
-            float m = 0.f;
-#pragma unroll
-            for (int i = 0; i < C; ++i) m = fmaxf(m, fabsf(g[i]));
-            // 2^(127 - e) for the exponent field e of the largest
-            const int e = max(254 - (int)(__float_as_uint(m) >> 23), 1);
-            const float sc = __uint_as_float((unsigned)e << 23);
-            unit = __longlong_as_double((long long)(1023 + 2 * (127 - e)) << 52);
-#pragma unroll
-            for (int i = 0; i < C; ++i) {
-                const float q = g[i] * sc;
-                pair(w[i] * (q * q));
-            }
-        } else {
-            constexpr unsigned MIN = (127u - 100u) << 23, MAX = (127u + 100u) << 23;
-            float t[C];
-            bool out = false;
-#pragma unroll
-            for (int i = 0; i < C; ++i) {
-                t[i] = w[i] * (g[i] * g[i]);
-                out = out || (__float_as_uint(t[i]) - MIN > MAX - MIN && g[i] != 0.f);
-            }
-            if (!out) {
-#pragma unroll
-                for (int i = 0; i < C; ++i) pair(t[i]);
-            } else {
-#pragma unroll
-                for (int i = 0; i < C; ++i) far += (double)w[i] * ((double)g[i] * (double)g[i]);
-            }
-        }
-    }
     // (an infinite sum has no second part)
-    __device__ __forceinline__ double value() const
-    {
-        if constexpr (ALL) return unit * ((double)hi + (double)(fabsf(hi) < __int_as_float(0x7f800000) ? lo : 0.f));
-        else return (double)hi + (double)lo + far;
-    }
-};
+    const float inf = __int_as_float(0x7f800000);
+    return __longlong_as_double((long long)(1023 + 2 * (127 - f)) << 52) * ((double)hi + (double)(fabsf(hi) < inf ? lo : 0.f));
+}
 
 // The product's factors at one frequency: with s = +1, Y = (a x + b y, c x + d y) for
 // Z = (x, y), a = T.x + H.x, b = H.y - T.y, c = T.y + H.y, d = T.x - H.x; s = -1 swaps a
@@ -439,7 +404,8 @@ __device__ __forceinline__ void cc_body(const CurveDev &c, int mode, int discret
             const T lam = (T)sc->lambda, dtp = (T)sc->dtau * ((const T *)c.prec_imex)[col_mode(col, c.hs)];
             // sections whose loads are issued together, a group ahead of the stores
             constexpr int CH = EARLY ? E : 4;
-            TermSum<T, CH == E> sum;
+            double sum = 0.0;
+            T wk[EARLY ? E : 1];
             T rs[CH], w[CH], av[CH], uv[CH];
             auto fetch = [&](int r0) {
 #pragma unroll
@@ -455,7 +421,7 @@ __device__ __forceinline__ void cc_body(const CurveDev &c, int mode, int discret
             fetch(0);
 #pragma unroll
             for (int r0 = 0; r0 < E; r0 += CH) {
-                T rc[CH], wc[CH], ac[CH], uc[CH], gc[CH];
+                T rc[CH], wc[CH], ac[CH], uc[CH];
 #pragma unroll
                 for (int i = 0; i < CH; ++i) {
                     rc[i] = rs[i];
@@ -470,8 +436,12 @@ __device__ __forceinline__ void cc_body(const CurveDev &c, int mode, int discret
                     const bool interior = n > 0 && n < P;
                     const T y = rc[i] * get(r);
                     const T g = interior ? -(ac[i] + lam * y) : T(0);
-                    if constexpr (sizeof(T) == 8) sum.add(wc[i], g);
-                    else gc[i] = g;
+                    if constexpr (sizeof(T) == 8) {
+                        sum += wc[i] * (g * g);
+                    } else {   // v[r] has been read
+                        v[r].y = g;
+                        if (EARLY) wk[EARLY ? r : 0] = wc[i];
+                    }
                     if (step) {
                         const T un = uc[i] + dtp * g;   // the end rows unchanged (g = 0)
                         if (interior) U[n] = un;
@@ -480,9 +450,12 @@ __device__ __forceinline__ void cc_body(const CurveDev &c, int mode, int discret
                         G[n] = g;
                     }
                 }
-                if constexpr (sizeof(T) == 4) sum.add(wc, gc);
             }
-            partsum = (col_mode(col, c.hs) == 0 ? 1.0 : 2.0) * sum.value();
+            if constexpr (sizeof(T) == 4) {
+                auto weight = [&](int r) { return EARLY ? wk[EARLY ? r : 0] : tid + NT * r < ns ? tab(wt + tid + NT * r) : T(0); };
+                sum = sum_terms<E>(weight, [&](int r) { return v[r].y; });
+            }
+            partsum = (col_mode(col, c.hs) == 0 ? 1.0 : 2.0) * sum;
             if (!step) break;
             // the differences of the updated column: section n + 1 is the next lane's, for a
             // warp's last lane the next warp's first (through `edge`)
@@ -696,13 +669,13 @@ __global__ void __launch_bounds__(F::NT) k_cx(const __grid_constant__ CurveDev c
                 break;
             }
             const T lam = (T)sc->lambda, dtp = (T)sc->dtau * ((const T *)c.prec_imex)[col_mode(col, c.hs)];
-            TermSum<T, false> sum;
+            double sum = 0.0;
 #pragma unroll
             for (int r = 0; r < E; ++r) {
                 const int n = n0 + NT * r;
                 const bool interior = n > 0 && n < P;
                 const T g = interior ? -(a[r] + lam * y[r]) : T(0);
-                sum.add(n < ns ? wt[n] : T(0), g);
+                sum += (n < ns ? wt[n] : T(0)) * (g * g);
                 if (DEFER) {
                     u[r] += dtp * g;   // the end rows unchanged (g = 0)
                     if (interior) U[n] = u[r];
@@ -710,7 +683,7 @@ __global__ void __launch_bounds__(F::NT) k_cx(const __grid_constant__ CurveDev c
                     G[n] = g;
                 }
             }
-            partsum = (col_mode(col, c.hs) == 0 ? 1.0 : 2.0) * sum.value();
+            partsum = (col_mode(col, c.hs) == 0 ? 1.0 : 2.0) * sum;
             if constexpr (!DEFER) break;
 #pragma unroll
             for (int p = 0; p < CS; ++p) {
