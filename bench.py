@@ -67,6 +67,8 @@ BYTES = {"fp64": 8, "fp32": 4, "bf16x2": 4, "bf16x3": 4}
 KERNEL_SOURCES = {
     "rows": ["ks_device.cuh", "ks_kernels.cu", "ks_internal.h"],
     "rows_tc": ["ks_rows_tc.cu", "ks_device.cuh", "ks_internal.h"],
+    "rows_cm": ["ks_rows_cm.cu", "ks_rfft.cuh", "ks_device.cuh", "ks_internal.h"],
+    "column": ["ks_colconv.cu", "ks_rfft.cuh", "ks_device.cuh", "ks_internal.h"],
     "fft4": ["ks_fft4.cu", "ks_device.cuh", "ks_internal.h"],
 }
 
@@ -597,7 +599,7 @@ def run_curve(args):
     # and D) or the cluster form of an explicit s_transform
     one_launch = "dt_update" in prof and "dt_store" not in prof
     kernels = {}   # name -> (mean ms per launch, algorithmic bytes, algorithmic flops, traffic kind)
-    rows_kind = "rows_tc" if precision.startswith("bf16") else "rows"
+    rows_kind = "rows_tc" if precision.startswith("bf16") else "rows_cm" if form == "column" else "rows"
     if "rows" in prof:
         kernels["rows"] = (prof["rows"]["ms"] / prof["rows"]["launches"], 4.0 * N * b * spec.Ns,
                            (fx + fpw) * M, rows_kind)
@@ -613,7 +615,7 @@ def run_curve(args):
             kernels[key] = (prof[key]["ms"] / prof[key]["launches"], by, fl, "fft4")
     dom = max(kernels, key=lambda k: kernels[k][0])
     t_dom, by_dom, fl_dom, kind = kernels[dom]
-    kernel_names = {"rows": "row phase (k_rows%s)" % ("_tc" if rows_kind == "rows_tc" else "_cm" if form == "column" else ""),
+    kernel_names = {"rows": "row phase (k_%s)" % rows_kind,
                     "dt_update": ("both contractions and the update (%s)" % ("k_cc" if form == "column" else form)
                                   if one_launch else "update contraction (%s)" % form), "dt_store": "D_t u contraction (%s)" % form}
     ach = by_dom / (t_dom / 1e3) / 1e9
@@ -635,6 +637,8 @@ def run_curve(args):
     traf = None
     if dom == "rows":
         traf = recorded_traffic("rows:%s:N%d:Ns%d:%s" % (rows_kind, N, spec.Ns, precision), rows_kind)
+    elif form == "column" and one_launch:
+        traf = recorded_traffic("both:column:N%d:Ns%d:%s" % (N, spec.Ns, precision), "column")
     elif form == "fft4" and not one_launch:
         traf = recorded_traffic("%s:fft4:N%d:Ns%d:%s" % (dom, N, spec.Ns, precision), "fft4")
     if traf:
